@@ -159,18 +159,20 @@ __device__ void batch_spread(const BatchDesc& D, int p, const qs_window& win, un
     }
     __syncthreads();
     const float inv_scale = s_scale[1];
-    for (int i = threadIdx.x; i < G; i += BT) grid[i] = (float)gridi[i] * inv_scale;
+    for (int i = threadIdx.x; i < G; i += BT) {
+        const int v = gridi[i];
+        __syncwarp();  // fft_cell moves cells within a warp's 32 only
+        fft_cell(grid, i) = (float)v * inv_scale;
+    }
     __syncthreads();
     const int Gh = G >> 1;
     const int log2n = 31 - __clz(Gh);
     float2* z = reinterpret_cast<float2*>(grid);
     fft_inplace<false>(z, Gh, log2n, D.tw, G);
-    real_filter<false>(z, Gh, D.D, D.tw);
+    real_filter<false>(z, z, Gh, log2n, D.D, D.tw);
     __syncthreads();
     fft_inplace<true>(z, Gh, log2n, D.tw, G);
-    float4* dst = reinterpret_cast<float4*>(D.H + (size_t)p * G);
-    const float4* src = reinterpret_cast<const float4*>(grid);
-    for (int i = threadIdx.x; i < (G >> 2); i += BT) dst[i] = src[i];
+    fft_store(grid, D.H + (size_t)p * G, G, 0);
 }
 
 template <int W>

@@ -8,47 +8,149 @@
 namespace qsdev {
 
 // ---------------------------------------------------------------------------
-// In-place radix-2 complex FFT of length n = G/2 in shared memory.
-// Forward uses e^{-2 pi i j / len}, inverse e^{+...}; both unnormalised.
-// tw[t] = e^{-2 pi i t / G}, t < G/2.
+// Complex FFT of length n = G/2 in place in shared memory, n a power of two.
+// Forward (e^{-2 pi i j / len}): decimation in frequency, natural order in,
+// digit-reversed order out; inverse (e^{+...}): the same passes backwards,
+// digit-reversed in, natural out, so that no pass reorders anything -- the
+// spectrum is only ever touched by real_filter, which goes through
+// fft_pos.  Both unnormalised.  tw[t] = e^{-2 pi i t / G}, t < G/2.
+//
+// The passes are bound by their barriers and shared-memory round trips, not
+// by arithmetic, so each takes eight points per thread (radix 8, after one
+// radix-2 or radix-4 pass when log2 n is no multiple of 3): ceil(log2 n / 3)
+// passes instead of the log2 n of a radix-2 transform and no bit reversal.
+// Element i lies at fft_sw(i): the XOR spreads the strides of 8 and 64
+// elements of the last passes over the banks without padding.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float2 cmul(float2 a, float2 b)
 {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+__device__ __forceinline__ int fft_sw(int i) { return i ^ ((i >> 4) & 15); }
+
+// Place of frequency k after the forward transform (before fft_sw).
+__device__ __forceinline__ int fft_pos(int k, int log2n)
+{
+    const int r = log2n % 3;
+    int len = (1 << log2n) >> r;
+    int pos = (k & ((1 << r) - 1)) * len;
+    k >>= r;
+    while (len > 1) {
+        len >>= 3;
+        pos += (k & 7) * len;
+        k >>= 3;
+    }
+    return pos;
+}
+
+template <bool INV>
+__device__ __forceinline__ float2 fft_rot(float2 a)  // times -i, inverse: +i
+{
+    return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+}
+
+template <bool INV>
+__device__ __forceinline__ void dft4(float2& a, float2& b, float2& c, float2& d)  // natural order in and out
+{
+    const float2 s0 = make_float2(a.x + c.x, a.y + c.y), d0 = make_float2(a.x - c.x, a.y - c.y);
+    const float2 s1 = make_float2(b.x + d.x, b.y + d.y);
+    const float2 d1 = fft_rot<INV>(make_float2(b.x - d.x, b.y - d.y));
+    a = make_float2(s0.x + s1.x, s0.y + s1.y);
+    b = make_float2(d0.x + d1.x, d0.y + d1.y);
+    c = make_float2(s0.x - s1.x, s0.y - s1.y);
+    d = make_float2(d0.x - d1.x, d0.y - d1.y);
+}
+
+template <bool INV, int R>
+__device__ __forceinline__ void dft_r(float2 (&v)[R])
+{
+    if constexpr (R == 2) {
+        const float2 t = make_float2(v[0].x - v[1].x, v[0].y - v[1].y);
+        v[0] = make_float2(v[0].x + v[1].x, v[0].y + v[1].y);
+        v[1] = t;
+    } else if constexpr (R == 4) {
+        dft4<INV>(v[0], v[1], v[2], v[3]);
+    } else {
+        dft4<INV>(v[0], v[2], v[4], v[6]);
+        dft4<INV>(v[1], v[3], v[5], v[7]);
+        constexpr float h = 0.70710678118654752440f;
+        const float2 e[4] = {v[0], v[2], v[4], v[6]};
+        float2 o[4] = {v[1], v[3], v[5], v[7]};
+        o[1] = INV ? make_float2(h * (o[1].x - o[1].y), h * (o[1].x + o[1].y))
+                   : make_float2(h * (o[1].x + o[1].y), h * (o[1].y - o[1].x));
+        o[2] = fft_rot<INV>(o[2]);
+        o[3] = INV ? make_float2(-h * (o[3].x + o[3].y), h * (o[3].x - o[3].y))
+                   : make_float2(h * (o[3].y - o[3].x), -h * (o[3].x + o[3].y));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = make_float2(e[k].x + o[k].x, e[k].y + o[k].y);
+            v[k + 4] = make_float2(e[k].x - o[k].x, e[k].y - o[k].y);
+        }
+    }
+}
+
+// One pass over all blocks of `len` elements; ends with a barrier.
+template <bool INV, int R>
+__device__ __forceinline__ void fft_pass(float2* z, int n, int len, const float2* __restrict__ tw, int G)
+{
+    constexpr int LR = R == 2 ? 1 : (R == 4 ? 2 : 3);
+    const int sub = len >> LR;
+    const int ts = G / len;
+    for (int b = threadIdx.x; b < (n >> LR); b += blockDim.x) {
+        const int j = b & (sub - 1);
+        const int base = ((b - j) << LR) + j;
+        float2 v[R], w[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = z[fft_sw(base + q * sub)];
+        if (sub > 1) {
+            // w^q from the table for q = 1, 2, 4 (indices below G/2), the others by one product
+            w[1] = __ldg(&tw[j * ts]);
+            if (R > 2) {
+                w[2] = __ldg(&tw[2 * j * ts]);
+                w[3] = cmul(w[1], w[2]);
+            }
+            if constexpr (R == 8) {
+                w[4] = __ldg(&tw[4 * j * ts]);
+                w[5] = cmul(w[1], w[4]);
+                w[6] = cmul(w[2], w[4]);
+                w[7] = cmul(w[3], w[4]);
+            }
+        }
+        if (INV && sub > 1) {
+#pragma unroll
+            for (int q = 1; q < R; ++q) v[q] = cmul(v[q], make_float2(w[q].x, -w[q].y));
+        }
+        dft_r<INV, R>(v);
+        if (!INV && sub > 1) {
+#pragma unroll
+            for (int q = 1; q < R; ++q) v[q] = cmul(v[q], w[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q) z[fft_sw(base + q * sub)] = v[q];
+    }
+    __syncthreads();
+}
+
+// The barrier before the first pass is the caller's.
 template <bool INV>
 __device__ inline void fft_inplace(float2* z, int n, int log2n, const float2* __restrict__ tw, int G)
 {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int j = (int)(__brev((unsigned)i) >> (32 - log2n));
-        if (j > i) {
-            const float2 t = z[i];
-            z[i] = z[j];
-            z[j] = t;
-        }
-    }
-    __syncthreads();
-    for (int len = 2; len <= n; len <<= 1) {
-        const int half = len >> 1;
-        const int stride = G / len;
-        for (int b = threadIdx.x; b < (n >> 1); b += blockDim.x) {
-            const int pos = b & (half - 1);
-            const int i = ((b - pos) << 1) + pos;
-            const int j = i + half;
-            float2 wv = __ldg(&tw[pos * stride]);
-            if (INV) wv.y = -wv.y;
-            const float2 a = z[i];
-            const float2 t = cmul(z[j], wv);
-            z[i] = make_float2(a.x + t.x, a.y + t.y);
-            z[j] = make_float2(a.x - t.x, a.y - t.y);
-        }
-        __syncthreads();
+    const int r = log2n % 3;
+    if (!INV) {
+        if (r == 1) fft_pass<false, 2>(z, n, n, tw, G);
+        else if (r == 2) fft_pass<false, 4>(z, n, n, tw, G);
+        for (int len = n >> r; len > 1; len >>= 3) fft_pass<false, 8>(z, n, len, tw, G);
+    } else {
+        for (int len = 8; len <= (n >> r); len <<= 3) fft_pass<true, 8>(z, n, len, tw, G);
+        if (r == 1) fft_pass<true, 2>(z, n, n, tw, G);
+        else if (r == 2) fft_pass<true, 4>(z, n, n, tw, G);
     }
 }
 
 // Real-input FFT post-processing, filter by D, and pre-processing of the
-// real-output inverse, all on the packed spectrum z (length Gh = G/2):
+// real-output inverse, all on the packed spectrum z (length Gh = G/2, in the
+// forward transform's order):
 //   z_j = g_{2j} + i g_{2j+1},  Z = FFT_Gh(z)
 //   X_k = (Z_k + conj Z_{Gh-k})/2 + e^{-2 pi i k/G} (Z_k - conj Z_{Gh-k})/(2i)   (k = 0..Gh)
 //   Y_k = D_k X_k
@@ -56,25 +158,28 @@ __device__ inline void fft_inplace(float2* z, int n, int log2n, const float2* __
 // so that IFFT_Gh(Z') interleaves the real sequence h_l = sum_k Y_k e^{2 pi i k l/G}.
 // DERIV: the filter is i g_k with the real table g (derivative coefficients
 // 2 pi i k c_k over psi^2), i.e. Y_k = i g_k X_k.
+// zo: where Z' is written (z itself, or a second buffer).
 template <bool DERIV>
-__device__ inline void real_filter(float2* z, int Gh, const float* __restrict__ D, const float2* __restrict__ tw)
+__device__ inline void real_filter(const float2* z, float2* zo, int Gh, int log2n, const float* __restrict__ D,
+                                   const float2* __restrict__ tw)
 {
     for (int k = threadIdx.x; k <= (Gh >> 1); k += blockDim.x) {
         if (k == 0) {
             const float2 z0 = z[0];
             if (DERIV) {
                 // g_0 = 0 and g_{Gh} = 0 (Gh > N_ft/2): the real parts at k = 0, Gh vanish
-                z[0] = make_float2(0.0f, 0.0f);
+                zo[0] = make_float2(0.0f, 0.0f);
                 continue;
             }
             const float y0 = __ldg(&D[0]) * (z0.x + z0.y);
             const float yh = __ldg(&D[Gh]) * (z0.x - z0.y);
-            z[0] = make_float2(y0 + yh, y0 - yh);
+            zo[0] = make_float2(y0 + yh, y0 - yh);
             continue;
         }
         const int k2 = Gh - k;
-        const float2 zk = z[k];
-        const float2 zc = make_float2(z[k2].x, -z[k2].y);  // conj Z_{Gh-k}
+        const int i1 = fft_sw(fft_pos(k, log2n)), i2 = fft_sw(fft_pos(k2, log2n));
+        const float2 zk = z[i1];
+        const float2 zc = make_float2(z[i2].x, -z[i2].y);  // conj Z_{Gh-k}
         const float2 A = make_float2(0.5f * (zk.x + zc.x), 0.5f * (zk.y + zc.y));
         const float2 B = make_float2(0.5f * (zk.y - zc.y), -0.5f * (zk.x - zc.x));  // -i (Zk - Zc)/2
         const float2 t = __ldg(&tw[k]);
@@ -91,16 +196,28 @@ __device__ inline void real_filter(float2* z, int Gh, const float* __restrict__ 
             const float2 sum = make_float2(Yk.x + Yk2.x, Yk.y - Yk2.y);
             const float2 dif = make_float2(Yk.x - Yk2.x, Yk.y + Yk2.y);
             const float2 r = cmul(tc, dif);
-            z[k] = make_float2(sum.x - r.y, sum.y + r.x);
+            zo[i1] = make_float2(sum.x - r.y, sum.y + r.x);
         }
         // Z'_{k2} = (Yk2 + conj Yk) + i (-t) (Yk2 - conj Yk)
         {
             const float2 sum = make_float2(Yk2.x + Yk.x, Yk2.y - Yk.y);
             const float2 dif = make_float2(Yk2.x - Yk.x, Yk2.y + Yk.y);
             const float2 r = cmul(make_float2(-t.x, -t.y), dif);
-            z[k2] = make_float2(sum.x - r.y, sum.y + r.x);
+            zo[i2] = make_float2(sum.x - r.y, sum.y + r.x);
         }
     }
+}
+
+// Grid cell c of the real sequence in the transform's buffer.
+__device__ __forceinline__ float& fft_cell(float* grid, int c) { return grid[2 * fft_sw(c >> 1) + (c & 1)]; }
+
+// Copy the inverse transform's G cells to global memory: dst[c] = cell (c + shift) mod G, shift even.
+__device__ __forceinline__ void fft_store(const float* grid, float* dst, int G, int shift)
+{
+    const float2* z = reinterpret_cast<const float2*>(grid);
+    float2* out = reinterpret_cast<float2*>(dst);
+    const int Gh = G >> 1, hs = shift >> 1;
+    for (int i = threadIdx.x; i < Gh; i += blockDim.x) out[i] = z[fft_sw((i + hs) & (Gh - 1))];
 }
 
 constexpr int IT_THREADS = 256;

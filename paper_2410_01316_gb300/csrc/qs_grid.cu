@@ -225,13 +225,10 @@ __device__ __forceinline__ void filter_store(const qs_launch& L, float* grid, in
     const int log2n = 31 - __clz(Gh);
     float2* z = reinterpret_cast<float2*>(grid);
     fft_inplace<false>(z, Gh, log2n, L.tw, G);
-    real_filter<false>(z, Gh, L.D, L.tw);
+    real_filter<false>(z, z, Gh, log2n, L.D, L.tw);
     __syncthreads();
     fft_inplace<true>(z, Gh, log2n, L.tw, G);
-    float4* dst = reinterpret_cast<float4*>(L.H + (size_t)p * G);
-    const float4* src = reinterpret_cast<const float4*>(grid);
-    const int hq = H >> 2, qmask = (G >> 2) - 1;
-    for (int i = threadIdx.x; i < (G >> 2); i += blockDim.x) dst[i] = src[(i + hq) & qmask];
+    fft_store(grid, L.H + (size_t)p * G, G, H);
 }
 
 template <int W, bool FUSED, int MODE, int PARAM, int PF>
@@ -335,7 +332,8 @@ __global__ void __launch_bounds__(256) spread_filter_kernel(qs_launch L, const f
             v += gridi[c * cstride + i];
             if (i < SPREAD_PAD) v += gridi[c * cstride + G + i];
         }
-        grid[i] = (float)v * inv_scale;
+        __syncwarp();  // fft_cell moves cells within a warp's 32 only
+        fft_cell(grid, i) = (float)v * inv_scale;
     }
     __syncthreads();
     filter_store(L, grid, p, H);
@@ -540,7 +538,7 @@ __device__ __forceinline__ void moment_grid(const qs_launch& L, const float* __r
             for (int j = 0; j < W; ++j) f += vtab[(G + c - j) * KS + j];
             v += f;
         }
-        grid[c] = v * inv_scale;
+        fft_cell(grid, c) = v * inv_scale;
     }
     __syncthreads();
 }
@@ -592,29 +590,21 @@ __device__ __forceinline__ void grad_filter_store(const qs_launch& L, float* gri
     const int log2n = 31 - __clz(Gh);
     float2* z = reinterpret_cast<float2*>(grid);
     float2* z2 = reinterpret_cast<float2*>(grid2);
-    const int hq = H >> 2, qmask = (G >> 2) - 1;
     fft_inplace<false>(z, Gh, log2n, L.tw, G);
     if (MODE == 2) {
-        for (int i = threadIdx.x; i < Gh; i += blockDim.x) z2[i] = z[i];
+        real_filter<true>(z, z2, Gh, log2n, Dd, L.tw);
         __syncthreads();
-        real_filter<false>(z, Gh, L.D, L.tw);
-        real_filter<true>(z2, Gh, Dd, L.tw);
+        real_filter<false>(z, z, Gh, log2n, L.D, L.tw);
         __syncthreads();
         fft_inplace<true>(z, Gh, log2n, L.tw, G);
         fft_inplace<true>(z2, Gh, log2n, L.tw, G);
-        float4* dst = reinterpret_cast<float4*>(L.H + (size_t)p * G);
-        const float4* src = reinterpret_cast<const float4*>(grid);
-        for (int i = threadIdx.x; i < (G >> 2); i += blockDim.x) dst[i] = src[(i + hq) & qmask];
-        float4* dst2 = reinterpret_cast<float4*>(H2 + (size_t)p * G);
-        const float4* src2 = reinterpret_cast<const float4*>(grid2);
-        for (int i = threadIdx.x; i < (G >> 2); i += blockDim.x) dst2[i] = src2[(i + hq) & qmask];
+        fft_store(grid, L.H + (size_t)p * G, G, H);
+        fft_store(grid2, H2 + (size_t)p * G, G, H);
     } else {
-        real_filter<true>(z, Gh, Dd, L.tw);
+        real_filter<true>(z, z, Gh, log2n, Dd, L.tw);
         __syncthreads();
         fft_inplace<true>(z, Gh, log2n, L.tw, G);
-        float4* dst2 = reinterpret_cast<float4*>(H2 + (size_t)p * G);
-        const float4* src = reinterpret_cast<const float4*>(grid);
-        for (int i = threadIdx.x; i < (G >> 2); i += blockDim.x) dst2[i] = src[(i + hq) & qmask];
+        fft_store(grid, H2 + (size_t)p * G, G, H);
     }
 }
 
@@ -645,7 +635,8 @@ __global__ void __launch_bounds__(256) spread_grad_kernel(qs_launch L, const flo
     __syncthreads();
     for (int i = threadIdx.x; i < G; i += blockDim.x) {
         const int v = gridi[i] + (i < SPREAD_PAD ? gridi[G + i] : 0);
-        grid[i] = (float)v * inv_scale;
+        __syncwarp();  // fft_cell moves cells within a warp's 32 only
+        fft_cell(grid, i) = (float)v * inv_scale;
     }
     __syncthreads();
     grad_filter_store<MODE>(L, grid, grid2, Dd, H2, p, H);
