@@ -7,6 +7,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "qmcslice.h"
@@ -33,6 +34,14 @@ constexpr int QS_GRAD_MAX_D = 32;              // largest d of the fused form's 
 constexpr int QS_BATCH_MAX_D = 64;             // largest d of a batched problem
 constexpr int QS_SOBOL_MAX_D = 4096;           // largest d of the Sobol' directions
 constexpr int QS_BATCH_STREAMS = 8;            // streams of a batch's concurrent mode
+
+// Slice-per-lane grid kernels (qs_lane.cu): the default window width only.
+constexpr int QS_LANE_W = 8;
+constexpr int QS_LANE_CTAS = 152;              // CTAs that the work is cut into: one per SM
+constexpr int64_t QS_LANE_MIN_PAIRS = 1 << 20;
+constexpr int QS_PREP_BLOCKS = 152;            // most blocks of the weight bound
+// wscale: scale, inverse, max |w| scale, non-finite; 2 partials per block; the ticket
+constexpr int QS_WSCALE_FLOATS = 4 + 2 * QS_PREP_BLOCKS + 4;
 
 // Spread kernel variants, in two families fixed by (G, W): the moment family
 // where its table fits two CTAs per SM, the tap family otherwise.  Within a
@@ -98,8 +107,10 @@ struct qs_launch {
     float* U;             // P x ldU projections (unfused forms)
     float* part;          // 2 x S x M partial slice sums (hi, lo)
     int S;                // number of slice groups of the interpolation
+    void* Qlo;            // low BF16 parts of the derivative values (tensor-core forms), [p / 32][m][32]
+    int lane_T;           // targets per CTA of the slice-per-lane interpolation
     unsigned int* flag;   // device error flag
-    float* wscale;        // [0] = 2^30 / sum|w| (fixed-point scale of the grids), [1] = its inverse
+    float* wscale;        // [0] = 2^30 / sum|w| (fixed-point scale of the grids), [1] = its inverse; QS_WSCALE_FLOATS
     int spread_variant;   // QS_SPREAD_* (all variants give bitwise identical grids)
     qs_window win;
     // tap polynomials in monomials of t = 2 s: tap_j(t) = sum_k atab[j K + k] t^k, K = qs_moment_count(W)
@@ -132,7 +143,7 @@ struct qs_plan_s {
     float* d_H;
     float* d_part;
     unsigned int* d_flag;
-    float* d_wscale;      // 2 floats, written by the weight-bound kernel of each sum
+    float* d_wscale;      // QS_WSCALE_FLOATS, written by the weight-bound kernel of each sum
     // gradients: derivative filter, second grid; per-component partials (fused form, d <= 32)
     float* d_Dd;          // G/2 + 1
     float* d_H2;          // P x G
@@ -157,6 +168,11 @@ struct qs_plan_s {
     // directions hi/lo (128-row boxes, the SM-pair kernel)
     alignas(64) unsigned char tmaps[6][128];
     alignas(64) unsigned char tmaps_y[6][128];  // the same with the targets' staging as A
+    // back-projection GEMM of the tensor-core forms: low parts of the derivative values, directions
+    // transposed and split (NULL: not available, the SIMT back-projection is used)
+    void* d_qlo;
+    void* d_xit;
+    alignas(64) unsigned char tmaps_q[6][128];
     bool gemm_pair;       // projection GEMM on SM pairs (cta_group::2)
     // qs_sum's fork: the targets' operand split runs on side_st during the sources' GEMM;
     // sev = fork, join (no timing), split start, split end (timing, read by qs_stage_times)
@@ -293,6 +309,15 @@ cudaError_t qs_launch_reduce_grad(const float* part, int S, int64_t M, int d, fl
 cudaError_t qs_launch_interp_deriv(const qs_launch& L, int W, const float* Hd, cudaStream_t st);
 cudaError_t qs_launch_backproj(const float* Q, int64_t ldQ, int64_t M, int P, const float* xi, int d, float scale,
                                const float* fac, float* out, cudaStream_t st);
+// The same on the tensor cores, from the BF16 parts that the slice-per-lane kernels write (maps from
+// qs_make_backproj_maps): M targets, inner dimension P.
+cudaError_t qs_launch_backproj_tc(const void* maps, int64_t M, int P, int d, float scale, const float* fac, float* out,
+                                  unsigned int* flag, cudaStream_t st);
+// U: [P / 32 rounded up][ldU][32] floats holding high and middle parts, qlo: the low parts, xit: three planes
+// of d rows of ldq BF16 (the directions transposed and split, qs_launch_split_xit).  maps: 6 x 128 bytes.
+bool qs_make_backproj_maps(unsigned char (*maps)[128], const float* U, const void* qlo, const void* xit, int64_t ldU,
+                           int P, int d, int ldq);
+cudaError_t qs_launch_split_xit(const float* xi, int P, int d, int ldq, void* xit, cudaStream_t st);
 bool qs_make_tmap(void* map_out, const void* base, int elem_bytes, int d, int64_t rows, int ldk, int box_rows);
 // max_blocks > 0 caps the grid (a split running beside another kernel).
 cudaError_t qs_launch_split_bf16(const float* X, int64_t rows, int d, int ldk, void* hi, void* lo, cudaStream_t st,
@@ -302,8 +327,9 @@ cudaError_t qs_launch_round_tf32(const float* X, int64_t rows, int d, int ldk, f
 // Rows [n_base, n_base + N) of the staged operands into columns [n_base, n_base + N) of U;
 // n_base a multiple of 128.
 // pair: the SM-pair (cta_group::2) kernel, which needs maps 4 / 5 and qs_tc_pair_available.
+// lanes: U[p / 32][n][32] (rows p / 32 of ldU points), all 32 slices of a group, instead of U[p][n].
 cudaError_t qs_launch_project_tc(int kind, const void* maps, int64_t n_base, int64_t N, int d, int P, float* U,
-                                 int64_t ldU, unsigned int* flag, cudaStream_t st, bool pair);
+                                 int64_t ldU, unsigned int* flag, cudaStream_t st, bool pair, bool lanes = false);
 bool qs_tc_pair_available(int kind);
 int qs_tc_pair_ctas(int kind);  // CTAs of a full-size SM-pair launch (2 x resident clusters)
 cudaError_t qs_launch_weight_scale(const qs_launch& L, const float* w, cudaStream_t st);
@@ -311,3 +337,31 @@ cudaError_t qs_launch_spread(const qs_launch& L, int W, const float* x, const fl
                              cudaStream_t st);
 cudaError_t qs_launch_interp(const qs_launch& L, int W, const float* y, bool fused, cudaStream_t st);
 cudaError_t qs_launch_reduce(const qs_launch& L, float* s, cudaStream_t st);
+
+// Slice-per-lane grid stages (qs_lane.cu).  grid: P x G, cleared and later holding the integer
+// grids (spread), filtered in place.  from_u: projections in L.U, U[p / 32][n][32]; otherwise
+// FP32 projections of x / y formed in the kernels (d <= QS_FUSED_MAX_D).
+cudaError_t qs_launch_lane_prep(const qs_launch& L, const float* w, float* grid, cudaStream_t st);
+cudaError_t qs_launch_lane_spread(const qs_launch& L, const float* x, const float* w, bool from_u, float* grid,
+                                  cudaStream_t st);
+// mode 0: plain filter in place; 1: derivative filter in place; 2: plain in place, derivative into H2
+cudaError_t qs_launch_lane_filter(const qs_launch& L, int mode, float* grid, const float* Dd, float* H2,
+                                  cudaStream_t st);
+// Slice sums of the rows H into L.part (L.S groups), or (deriv) the values for the back-projection: FP32 into
+// L.U, U[p][m]; tensor-core forms as BF16 parts into L.U and L.Qlo.
+cudaError_t qs_launch_lane_interp(const qs_launch& L, const float* y, bool from_u, const float* H, bool deriv,
+                                  cudaStream_t st);
+void qs_lane_shape(int64_t M, int P, int S_max, int* T, int* S);
+// Whether the grid stages of n points and P slices run slice-per-lane: the default window, a form whose
+// projections they can take, enough (point, slice) pairs to fill the SMs, and windows that are likely to
+// fit one walk.  The projections of points within R / 2 span G tau R cells, and about 8.4 standard
+// deviations of (G tau R / 2) / sqrt(d) of them in high dimensions; the shared memory holds some 1400
+// (two walks take 2.8 ms where the point-per-lane kernels take 1.9: d = 3, 2 x 1.5e5 points, P = 1024,
+// G = 4096).
+inline bool qs_lane_use(qs_proj proj, int W, int d, int64_t n, int P, double span)
+{
+    if (W != QS_LANE_W || (proj == QS_PROJ_FP32 && d > QS_FUSED_MAX_D)) return false;
+    const double sigmas = 4.2 / sqrt((double)d);
+    if (span * (sigmas < 1.0 ? sigmas : 1.0) > 1600.0) return false;
+    return n >= 512 && n < ((int64_t)1 << 31) && n * (int64_t)P >= QS_LANE_MIN_PAIRS;
+}

@@ -208,7 +208,7 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     int64_t S = (1024 + blocks_m - 1) / blocks_m;
     if (S > S_max) S = S_max;
     if (S < 1) S = 1;
-    const size_t o_flag = 0, o_wscale = 256, o_psihat = 512;
+    const size_t o_flag = 0, o_wscale = 256, o_psihat = o_wscale + align256(QS_WSCALE_FLOATS * 4);
     const size_t o_c = o_psihat + align256((size_t)(K + 1) * 8);
     const size_t o_D = o_c + align256((size_t)D.n_ft * 8);
     const size_t o_tw = o_D + align256((size_t)(G / 2 + 1) * 4);
@@ -217,6 +217,17 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     const size_t o_part = o_H + align256((size_t)P * G * 4);
     const size_t avail = o_part < QS_NOALLOC_SCRATCH_BYTES ? QS_NOALLOC_SCRATCH_BYTES - o_part : 0;
     while (S > 1 && (size_t)(2 * S) * (size_t)M * 4 > avail) --S;
+    // the slice-per-lane kernels by the rule of qs_sum, with as many slice groups as the scratch holds
+    const double span = G * qs_tau_rule(D.kernel, D.kparam, D.radius) * D.radius;
+    const bool lx = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, N, P, span),
+               ly = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, M, P, span);
+    int lane_T = 0;
+    if (ly) {
+        int lane_S = 1;
+        int64_t fit = (int64_t)(avail / 8) / M;
+        qs_lane_shape(M, P, (int)(fit < 1 ? 1 : (fit < S_max ? fit : S_max)), &lane_T, &lane_S);
+        S = lane_S;
+    }
     const size_t need = o_part + (size_t)(2 * S) * (size_t)M * 4;
     if (need > QS_NOALLOC_SCRATCH_BYTES)
         return nfail(QS_ERR_UNSUPPORTED,
@@ -243,6 +254,7 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     L.half_G = 0.5f * (float)G;
     L.U = nullptr;
     L.S = (int)S;
+    L.lane_T = lane_T;
     L.spread_variant = qs_spread_default(G, W);
 
     unsigned char* base = nullptr;
@@ -268,7 +280,7 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     L.part = reinterpret_cast<float*>(base + o_part);
     L.flag = reinterpret_cast<unsigned int*>(base + o_flag);
     L.wscale = reinterpret_cast<float*>(base + o_wscale);
-    e = cudaMemsetAsync(base + o_flag, 0, sizeof(unsigned int), st);
+    e = cudaMemsetAsync(base + o_flag, 0, o_psihat, st);  // the flag, and the ticket of the weight bound
     if (e != cudaSuccess) return nfail(QS_ERR_CUDA, "qs_sum_noalloc: clear flag: %s", cudaGetErrorString(e));
     const int64_t nd = (int64_t)P * d;
     scale_dirs_kernel<<<(unsigned)((nd + 255) / 256), 256, 0, st>>>(dirs_dev, nd, (double)G * tau,
@@ -282,9 +294,16 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
         if (N == 0) {
             e = cudaMemsetAsync(s, 0, (size_t)M * sizeof(float), st);
         } else {
-            e = qs_launch_weight_scale(L, w, st);
-            if (e == cudaSuccess) e = qs_launch_spread(L, W, x, w, true, st);
-            if (e == cudaSuccess) e = qs_launch_interp(L, W, y, true, st);
+            if (lx) {
+                e = qs_launch_lane_prep(L, w, L.H, st);
+                if (e == cudaSuccess) e = qs_launch_lane_spread(L, x, w, false, L.H, st);
+                if (e == cudaSuccess) e = qs_launch_lane_filter(L, 0, L.H, nullptr, nullptr, st);
+            } else {
+                e = qs_launch_weight_scale(L, w, st);
+                if (e == cudaSuccess) e = qs_launch_spread(L, W, x, w, true, st);
+            }
+            if (e == cudaSuccess)
+                e = ly ? qs_launch_lane_interp(L, y, false, L.H, false, st) : qs_launch_interp(L, W, y, true, st);
             if (e == cudaSuccess) e = qs_launch_reduce(L, s, st);
         }
     }

@@ -200,7 +200,8 @@ void free_plan(qs_plan p)
     if (p->side_st) cudaStreamDestroy(p->side_st);
     void* bufs[] = {p->d_dirs, p->d_dirs_s, p->d_c, p->d_psihat, p->d_D, p->d_tw, p->d_U, p->d_H,
                     p->d_part, p->d_flag, p->d_wscale, p->d_x, p->d_w, p->d_y, p->d_s, p->d_xi_hi, p->d_xi_lo,
-                    p->d_xs_hi, p->d_xs_lo, p->d_ys_hi, p->d_ys_lo, p->d_Dd, p->d_H2, p->d_gpart, p->d_sortws};
+                    p->d_xs_hi, p->d_xs_lo, p->d_ys_hi, p->d_ys_lo, p->d_Dd, p->d_H2, p->d_gpart, p->d_sortws, p->d_qlo,
+                    p->d_xit};
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete p;
@@ -253,6 +254,21 @@ qs_launch make_launch(const qs_plan p, int64_t N, int64_t M, int64_t targets_per
     return L;
 }
 
+// Whether the grid stages of n points (sources or targets) run slice-per-lane.
+bool lane_use(const qs_plan p, int64_t n)
+{
+    return qs_lane_use(p->proj, p->W, p->desc.d, n, p->desc.P, p->G * p->tau * p->desc.radius);
+}
+
+bool tensor_form(const qs_plan p) { return p->proj == QS_PROJ_BF16X3 || p->proj == QS_PROJ_TF32; }
+
+// The same for the targets of a gradient, which the tensor-core forms back-project from BF16 parts.
+bool grad_lane(const qs_plan p, int64_t n) { return lane_use(p, n) && (!tensor_form(p) || p->d_qlo); }
+
+// The launch of the interpolation at M targets: lane_T and S of the slice-per-lane kernel, or S of the
+// point-per-lane one (make_launch's).
+void lane_launch(const qs_plan p, qs_launch* L) { qs_lane_shape(L->M, L->P, p->S_max, &L->lane_T, &L->S); }
+
 // Operand preparation of the tensor-core forms (BF16 hi/lo split or TF32
 // rounding of the points into the plan's staging: the targets' own staging
 // when ystage, so that it can run while the sources' GEMM reads theirs);
@@ -273,40 +289,44 @@ cudaError_t project_prep(const qs_plan p, const float* X, int64_t rows, cudaStre
     }
 }
 
-// The projection GEMM U = G tau X Xi^T (after project_prep for the tensor-core forms).
-cudaError_t project_gemm(const qs_plan p, const float* X, int64_t rows, cudaStream_t st, bool ystage = false)
+// The projection GEMM U = G tau X Xi^T (after project_prep for the tensor-core forms).  lanes: for the
+// slice-per-lane grid kernels, slice-interleaved; nothing for FP32, whose projections they form themselves.
+cudaError_t project_gemm(const qs_plan p, const float* X, int64_t rows, cudaStream_t st, bool ystage = false,
+                         bool lanes = false)
 {
     const int d = p->desc.d, P = p->desc.P;
     const void* maps = ystage ? (const void*)p->tmaps_y : (const void*)p->tmaps;
     switch (p->proj) {
-        case QS_PROJ_FP32: return qs_launch_project_fp32(X, rows, d, p->d_dirs_s, P, p->d_U, p->ldU, st);
+        case QS_PROJ_FP32:
+            return lanes ? cudaSuccess : qs_launch_project_fp32(X, rows, d, p->d_dirs_s, P, p->d_U, p->ldU, st);
         case QS_PROJ_BF16X3:
-            return qs_launch_project_tc(0, maps, 0, rows, d, P, p->d_U, p->ldU, p->d_flag, st, p->gemm_pair);
+            return qs_launch_project_tc(0, maps, 0, rows, d, P, p->d_U, p->ldU, p->d_flag, st, p->gemm_pair, lanes);
         case QS_PROJ_TF32:
-            return qs_launch_project_tc(1, maps, 0, rows, d, P, p->d_U, p->ldU, p->d_flag, st, p->gemm_pair);
+            return qs_launch_project_tc(1, maps, 0, rows, d, P, p->d_U, p->ldU, p->d_flag, st, p->gemm_pair, lanes);
         default: return cudaErrorInvalidValue;
     }
 }
 
 // Rows [r0, r0 + rows) of X (N x d, row-major) projected into columns
 // [r0, r0 + rows) of U, operand preparation included; r0 a multiple of 128.
-cudaError_t project_rows(const qs_plan p, const float* X, int64_t r0, int64_t rows, cudaStream_t st)
+cudaError_t project_rows(const qs_plan p, const float* X, int64_t r0, int64_t rows, cudaStream_t st, bool lanes)
 {
     const int d = p->desc.d, P = p->desc.P;
     const float* Xr = X + r0 * d;
     cudaError_t e;
     switch (p->proj) {
-        case QS_PROJ_FP32: return qs_launch_project_fp32(Xr, rows, d, p->d_dirs_s, P, p->d_U + r0, p->ldU, st);
+        case QS_PROJ_FP32:
+            return lanes ? cudaSuccess : qs_launch_project_fp32(Xr, rows, d, p->d_dirs_s, P, p->d_U + r0, p->ldU, st);
         case QS_PROJ_BF16X3:
             e = qs_launch_split_bf16(Xr, rows, d, p->ldk, (uint16_t*)p->d_xs_hi + r0 * p->ldk,
                                      (uint16_t*)p->d_xs_lo + r0 * p->ldk, st);
             return e == cudaSuccess ? qs_launch_project_tc(0, p->tmaps, r0, rows, d, P, p->d_U, p->ldU, p->d_flag, st,
-                                                           p->gemm_pair)
+                                                           p->gemm_pair, lanes)
                                     : e;
         case QS_PROJ_TF32:
             e = qs_launch_round_tf32(Xr, rows, d, p->ldk, (float*)p->d_xs_hi + r0 * p->ldk, st);
             return e == cudaSuccess ? qs_launch_project_tc(1, p->tmaps, r0, rows, d, P, p->d_U, p->ldU, p->d_flag, st,
-                                                           p->gemm_pair)
+                                                           p->gemm_pair, lanes)
                                     : e;
         default: return cudaErrorInvalidValue;
     }
@@ -322,10 +342,10 @@ int64_t host_chunk_rows(int64_t n, int64_t unit = 128, int chunks = QS_HOST_CHUN
 }
 
 // U = G tau X Xi^T for the plan's projection form.
-cudaError_t project(const qs_plan p, const float* X, int64_t rows, cudaStream_t st)
+cudaError_t project(const qs_plan p, const float* X, int64_t rows, cudaStream_t st, bool lanes = false)
 {
     cudaError_t e = project_prep(p, X, rows, st);
-    return e == cudaSuccess ? project_gemm(p, X, rows, st) : e;
+    return e == cudaSuccess ? project_gemm(p, X, rows, st, false, lanes) : e;
 }
 
 }  // namespace
@@ -565,10 +585,10 @@ qs_status qs_plan_create(qs_plan* out, const qs_plan_desc* desc)
         QS_ALLOC(p->d_H2, (size_t)P * G);
     }
     QS_ALLOC(p->d_flag, 1);
-    QS_ALLOC(p->d_wscale, 2);
+    QS_ALLOC(p->d_wscale, QS_WSCALE_FLOATS);
     const bool tc = proj == QS_PROJ_BF16X3 || proj == QS_PROJ_TF32;
     if (proj == QS_PROJ_FP32 || tc) {
-        p->U_elems = (size_t)P * (size_t)p->ldU;
+        p->U_elems = (size_t)((P + 31) / 32 * 32) * (size_t)p->ldU;  // whole slice groups
         QS_ALLOC(p->d_U, p->U_elems);
     }
     const int64_t stage_rows = maxnm > 0 ? maxnm : 1;
@@ -620,6 +640,7 @@ qs_status qs_plan_create(qs_plan* out, const qs_plan_desc* desc)
              "copy window transform");
     QS_CHECK(cudaMemcpy(p->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice), "copy twiddles");
     QS_CHECK(cudaMemset(p->d_flag, 0, sizeof(unsigned int)), "clear flag");
+    QS_CHECK(cudaMemset(p->d_wscale, 0, QS_WSCALE_FLOATS * sizeof(float)), "clear weight-bound ticket");
     if (D.kernel == QS_RIESZ || D.kernel == QS_TPS) {
         // no classical transform: the periodised kernel's coefficients by host quadrature
         std::vector<double> ch;
@@ -663,6 +684,25 @@ qs_status qs_plan_create(qs_plan* out, const qs_plan_desc* desc)
         for (int i = 0; i < 4; ++i)
             QS_CHECK(cudaEventCreateWithFlags(&p->sev[i], i < 2 ? cudaEventDisableTiming : cudaEventDefault),
                      "fork / join events");
+        // back-projection GEMM: its buffers only make gradients faster, so a plan does without where they
+        // do not fit
+        if (W == QS_LANE_W) {
+            const size_t groups = (P + 31) / 32;
+            const int ldq = (P + 7) / 8 * 8;
+            uint16_t *ql = nullptr, *xt = nullptr;
+            bool okq = dalloc(&ql, groups * (size_t)p->ldU * 32) == cudaSuccess;
+            p->d_qlo = ql;
+            okq = okq && dalloc(&xt, (size_t)3 * d * ldq) == cudaSuccess;
+            p->d_xit = xt;
+            okq = okq && qs_make_backproj_maps(p->tmaps_q, p->d_U, ql, xt, p->ldU, P, d, ldq) &&
+                  qs_launch_split_xit(p->d_dirs, P, d, ldq, xt, 0) == cudaSuccess;
+            if (!okq) {
+                cudaGetLastError();
+                cudaFree(p->d_qlo);
+                cudaFree(p->d_xit);
+                p->d_qlo = p->d_xit = nullptr;
+            }
+        }
         // the SM-pair GEMM where the GEMM is tensor-bound (d >= 256: 6 d flop
         // per 4 B of U written) and two-CTA clusters of it can be resident;
         // below, the U stores bound both forms and the single-SM one is faster
@@ -733,6 +773,8 @@ qs_status qs_sum(qs_plan p, const float* x, int64_t N, const float* w, const flo
     }
     const bool fused = p->proj == QS_PROJ_FP32_FUSED;
     qs_launch L = make_launch(p, N, M, 256 * qs_interp_tpt(fused, p->desc.d, p->G));
+    const bool lx = lane_use(p, N), ly = lane_use(p, M), from_u = tensor_form(p);
+    if (ly) lane_launch(p, &L);
     const bool tm = p->timing != 0;
 #define QS_MARK(i)                                              \
     do {                                                        \
@@ -764,13 +806,19 @@ qs_status qs_sum(qs_plan p, const float* x, int64_t N, const float* w, const flo
         if (e != cudaSuccess) return cuda_fail(e, "qs_sum: operand split of y");
     }
     if (!fused) {
-        e = project_gemm(p, x, N, st);
+        e = project_gemm(p, x, N, st, false, lx);
         if (e != cudaSuccess) return cuda_fail(e, "qs_sum: projection of x");
     }
     QS_MARK(2);
-    e = qs_launch_weight_scale(L, w, st);
-    if (e != cudaSuccess) return cuda_fail(e, "qs_sum: weight bound");
-    e = qs_launch_spread(L, p->W, x, w, fused, st);
+    if (lx) {
+        e = qs_launch_lane_prep(L, w, p->d_H, st);
+        if (e == cudaSuccess) e = qs_launch_lane_spread(L, x, w, from_u, p->d_H, st);
+        if (e == cudaSuccess) e = qs_launch_lane_filter(L, 0, p->d_H, nullptr, nullptr, st);
+    } else {
+        e = qs_launch_weight_scale(L, w, st);
+        if (e != cudaSuccess) return cuda_fail(e, "qs_sum: weight bound");
+        e = qs_launch_spread(L, p->W, x, w, fused, st);
+    }
     if (e != cudaSuccess) return cuda_fail(e, "qs_sum: spread");
     QS_MARK(3);
     if (fork) {
@@ -782,11 +830,11 @@ qs_status qs_sum(qs_plan p, const float* x, int64_t N, const float* w, const flo
     }
     QS_MARK(4);
     if (!fused) {
-        e = project_gemm(p, y, M, st, fork);
+        e = project_gemm(p, y, M, st, fork, ly);
         if (e != cudaSuccess) return cuda_fail(e, "qs_sum: projection of y");
     }
     QS_MARK(5);
-    e = qs_launch_interp(L, p->W, y, fused, st);
+    e = ly ? qs_launch_lane_interp(L, y, from_u, p->d_H, false, st) : qs_launch_interp(L, p->W, y, fused, st);
     if (e != cudaSuccess) return cuda_fail(e, "qs_sum: interpolation");
     QS_MARK(6);
     e = qs_launch_reduce(L, s, st);
@@ -915,34 +963,61 @@ qs_status qs_grad(qs_plan p, const float* x, int64_t N, const float* w, const fl
     cudaStream_t st = (cudaStream_t)stream;
     const int d = p->desc.d;
     const float scale = (float)(p->tau / (double)p->desc.P);
-    // unfused plans project sources and targets with their GEMM into U first
-    const bool fused = p->proj == QS_PROJ_FP32_FUSED;
-    // unfused forms: the derivative values q_{m,p} are written over the
-    // projections in U and back-projected onto the directions by a GEMM (faster
-    // than d compensated sums per target-slice at any d: 2.07 against 2.36 ms per
-    // MMD-flow step at d = 16 with the 64-wide tile); the fused form has no U and
-    // keeps the per-component sums (d <= QS_GRAD_MAX_D)
-    const bool gemm_bp = !fused;
+    const bool fused = p->proj == QS_PROJ_FP32_FUSED, from_u = tensor_form(p);
+    // Sources -> grids: plain (into d_H) and / or derivative (into d_H2).
+    auto grids = [&](const qs_launch& L, const float* pts, const float* wt, bool plain, bool deriv) {
+        const bool lane = lane_use(p, L.N);
+        cudaError_t e = lane ? cudaSuccess : qs_launch_weight_scale(L, wt, st);
+        if (e == cudaSuccess && !fused) e = project(p, pts, L.N, st, lane);
+        if (e != cudaSuccess) return e;
+        if (!lane)
+            return deriv ? qs_launch_spread_grad(L, p->W, pts, wt, plain ? 2 : 1, fused, p->d_Dd, p->d_H2, st)
+                         : qs_launch_spread(L, p->W, pts, wt, fused, st);
+        float* grid = plain ? p->d_H : p->d_H2;
+        e = qs_launch_lane_prep(L, wt, grid, st);
+        if (e == cudaSuccess) e = qs_launch_lane_spread(L, pts, wt, from_u, grid, st);
+        return e == cudaSuccess ? qs_launch_lane_filter(L, plain && deriv ? 2 : (deriv ? 1 : 0), grid, p->d_Dd, p->d_H2, st)
+                                : e;
+    };
+    // Plain values of the grids at the targets (projected already where the form is unfused), summed over slices.
+    auto values = [&](qs_launch L, const float* pts, float* out) {
+        const bool lane = fused ? lane_use(p, L.M) : grad_lane(p, L.M);
+        if (lane) lane_launch(p, &L);
+        cudaError_t e = lane ? qs_launch_lane_interp(L, pts, from_u, p->d_H, false, st)
+                             : qs_launch_interp(L, p->W, pts, fused, st);
+        return e == cudaSuccess ? qs_launch_reduce(L, out, st) : e;
+    };
+    // Derivative values at the targets, back-projected onto the directions: out[m] = scale fac_m sum_p q_{m,p} xi_p.
+    // The unfused forms write q over the projections in U and back-project with a GEMM (faster than d
+    // compensated sums per target-slice at any d: 2.07 against 2.36 ms per MMD-flow step at d = 16 with
+    // the 64-wide tile); the fused form has no U and keeps the per-component sums (d <= QS_GRAD_MAX_D).
+    auto gradient = [&](qs_launch L, const float* pts, const float* fac, float* out) {
+        cudaError_t e;
+        if (fused) {
+            e = qs_launch_interp_grad(L, p->W, pts, p->d_H2, p->d_dirs, p->d_gpart, fused, st);
+            return e == cudaSuccess ? qs_launch_reduce_grad(p->d_gpart, L.S, L.M, d, scale, fac, out, st) : e;
+        }
+        if (!grad_lane(p, L.M)) {
+            cudaError_t e1 = qs_launch_interp_deriv(L, p->W, p->d_H2, st);
+            return e1 == cudaSuccess ? qs_launch_backproj(p->d_U, p->ldU, L.M, L.P, p->d_dirs, d, scale, fac, out, st) : e1;
+        }
+        qs_lane_shape(L.M, L.P, (L.P + 31) / 32, &L.lane_T, &L.S);  // no partial sums: any number of groups
+        L.Qlo = p->d_qlo;
+        e = qs_launch_lane_interp(L, pts, from_u, p->d_H2, true, st);
+        if (e != cudaSuccess) return e;
+        return from_u ? qs_launch_backproj_tc(p->tmaps_q, L.M, L.P, d, scale, fac, out, p->d_flag, st)
+                      : qs_launch_backproj(p->d_U, p->ldU, L.M, L.P, p->d_dirs, d, scale, fac, out, st);
+    };
     cudaError_t e = cudaSuccess;
     // dL/dy_m = (tau/P) v_m sum_p xi_p sum_n w_n g'(b_{m,p} - a_{n,p}): sources x, targets y
     if (gy && M > 0) {
         if (N == 0) {
             e = cudaMemsetAsync(gy, 0, (size_t)M * d * sizeof(float), st);
         } else {
-            qs_launch L = make_launch(p, N, M, 256);
-            e = qs_launch_weight_scale(L, w, st);
-            if (e == cudaSuccess && !fused) e = project(p, x, N, st);
-            if (e == cudaSuccess) e = qs_launch_spread_grad(L, p->W, x, w, 1, fused, p->d_Dd, p->d_H2, st);
-            if (e == cudaSuccess && !fused) e = project(p, y, M, st);
-            if (gemm_bp) {
-                if (e == cudaSuccess) e = qs_launch_interp_deriv(L, p->W, p->d_H2, st);
-                if (e == cudaSuccess)
-                    e = qs_launch_backproj(p->d_U, p->ldU, M, p->desc.P, p->d_dirs, d, scale, v, gy, st);
-            } else {
-                if (e == cudaSuccess)
-                    e = qs_launch_interp_grad(L, p->W, y, p->d_H2, p->d_dirs, p->d_gpart, fused, st);
-                if (e == cudaSuccess) e = qs_launch_reduce_grad(p->d_gpart, L.S, M, d, scale, v, gy, st);
-            }
+            const qs_launch L = make_launch(p, N, M, 256);
+            e = grids(L, x, w, false, true);
+            if (e == cudaSuccess && !fused) e = project(p, y, M, st, grad_lane(p, M));
+            if (e == cudaSuccess) e = gradient(L, y, v, gy);
         }
         if (e != cudaSuccess) return cuda_fail(e, "qs_grad: gradient in y");
     }
@@ -953,34 +1028,15 @@ qs_status qs_grad(qs_plan p, const float* x, int64_t N, const float* w, const fl
             if (gx) e = cudaMemsetAsync(gx, 0, (size_t)N * d * sizeof(float), st);
             if (e == cudaSuccess && gw) e = cudaMemsetAsync(gw, 0, (size_t)N * sizeof(float), st);
         } else {
-            // gw uses the (fused) interpolation kernel, gx the gradient kernel: each
+            // gw uses the interpolation kernel, gx the gradient kernel: each
             // gets the slice-group count matching its CTA shape
-            qs_launch L = make_launch(p, M, N, 256);
-            qs_launch Lw = make_launch(p, M, N, 256 * qs_interp_tpt(fused, p->desc.d, p->G));
-            e = qs_launch_weight_scale(L, v, st);
-            if (e == cudaSuccess && !fused) e = project(p, y, M, st);
-            if (e == cudaSuccess) {
-                if (gx)
-                    e = qs_launch_spread_grad(L, p->W, y, v, gw ? 2 : 1, fused, p->d_Dd, p->d_H2, st);
-                else
-                    e = qs_launch_spread(L, p->W, y, v, fused, st);
-            }
-            if (e == cudaSuccess && !fused) e = project(p, x, N, st);
-            if (gemm_bp) {
-                // the plain interpolation reads the projections before the
-                // derivative values overwrite them
-                if (e == cudaSuccess && gw) e = qs_launch_interp(Lw, p->W, x, fused, st);
-                if (e == cudaSuccess && gw) e = qs_launch_reduce(Lw, gw, st);
-                if (e == cudaSuccess && gx) e = qs_launch_interp_deriv(L, p->W, p->d_H2, st);
-                if (e == cudaSuccess && gx)
-                    e = qs_launch_backproj(p->d_U, p->ldU, N, p->desc.P, p->d_dirs, d, scale, w, gx, st);
-            } else {
-                if (e == cudaSuccess && gx)
-                    e = qs_launch_interp_grad(L, p->W, x, p->d_H2, p->d_dirs, p->d_gpart, fused, st);
-                if (e == cudaSuccess && gx) e = qs_launch_reduce_grad(p->d_gpart, L.S, N, d, scale, w, gx, st);
-                if (e == cudaSuccess && gw) e = qs_launch_interp(Lw, p->W, x, fused, st);
-                if (e == cudaSuccess && gw) e = qs_launch_reduce(Lw, gw, st);
-            }
+            const qs_launch L = make_launch(p, M, N, 256);
+            e = grids(L, y, v, gw != nullptr, gx != nullptr);
+            if (e == cudaSuccess && !fused) e = project(p, x, N, st, grad_lane(p, N));
+            // the plain interpolation reads the projections before the
+            // derivative values overwrite them
+            if (e == cudaSuccess && gw) e = values(make_launch(p, M, N, 256 * qs_interp_tpt(fused, d, p->G)), x, gw);
+            if (e == cudaSuccess && gx) e = gradient(L, x, w, gx);
         }
         if (e != cudaSuccess) return cuda_fail(e, "qs_grad: gradients in x / w");
     }
@@ -1196,8 +1252,13 @@ qs_status qs_sum_host(qs_plan p, const float* xh, int64_t N, const float* wh, co
         cudaEvent_t* ex = p->hev + 1;
         cudaEvent_t* ey = p->hev + 1 + QS_HOST_CHUNKS;
         const bool fused = p->proj == QS_PROJ_FP32_FUSED;
+        qs_launch L = make_launch(p, N, M, 256 * qs_interp_tpt(fused, d, p->G));
+        const bool lx = lane_use(p, N), ly = lane_use(p, M), from_u = tensor_form(p);
+        if (ly) lane_launch(p, &L);
+        // slice-per-lane interpolation: one launch once all targets are there, so that it fills the SMs;
+        // the chunks of y are only projected, and can be as many as those of x
         const int64_t cx = host_chunk_rows(N),
-                      cy = host_chunk_rows(M, 256 * qs_interp_tpt(fused, d, p->G), QS_HOST_Y_CHUNKS);
+                      cy = ly ? host_chunk_rows(M) : host_chunk_rows(M, 256 * qs_interp_tpt(fused, d, p->G), QS_HOST_Y_CHUNKS);
         const int nx = (int)((N + cx - 1) / cx), ny = (int)((M + cy - 1) / cy);
         // the copies wait for the work already queued on `stream` (it may read the staging buffers)
         e = cudaEventRecord(p->hev[0], st);
@@ -1214,28 +1275,35 @@ qs_status qs_sum_host(qs_plan p, const float* xh, int64_t N, const float* wh, co
             if (e == cudaSuccess) e = cudaEventRecord(ey[i], cs);
         }
         if (e != cudaSuccess) return cuda_fail(e, "qs_sum_host: copy in");
-        qs_launch L = make_launch(p, N, M, 256 * qs_interp_tpt(fused, d, p->G));
         if (fused) e = cudaStreamWaitEvent(st, ex[nx - 1], 0);
         for (int i = 0; !fused && e == cudaSuccess && i < nx; ++i) {
             const int64_t r0 = i * cx, r = (N - r0 < cx ? N - r0 : cx);
             e = cudaStreamWaitEvent(st, ex[i], 0);
-            if (e == cudaSuccess) e = project_rows(p, p->d_x, r0, r, st);
+            if (e == cudaSuccess) e = project_rows(p, p->d_x, r0, r, st, lx);
         }
         if (e != cudaSuccess) return cuda_fail(e, "qs_sum_host: projection of x");
-        e = qs_launch_weight_scale(L, wh ? p->d_w : nullptr, st);
-        if (e == cudaSuccess) e = qs_launch_spread(L, p->W, p->d_x, wh ? p->d_w : nullptr, fused, st);
+        const float* dw = wh ? p->d_w : nullptr;
+        if (lx) {
+            e = qs_launch_lane_prep(L, dw, p->d_H, st);
+            if (e == cudaSuccess) e = qs_launch_lane_spread(L, p->d_x, dw, from_u, p->d_H, st);
+            if (e == cudaSuccess) e = qs_launch_lane_filter(L, 0, p->d_H, nullptr, nullptr, st);
+        } else {
+            e = qs_launch_weight_scale(L, dw, st);
+            if (e == cudaSuccess) e = qs_launch_spread(L, p->W, p->d_x, dw, fused, st);
+        }
         if (e != cudaSuccess) return cuda_fail(e, "qs_sum_host: spread");
         for (int i = 0; e == cudaSuccess && i < ny; ++i) {
             const int64_t r0 = i * cy, r = (M - r0 < cy ? M - r0 : cy);
             e = cudaStreamWaitEvent(st, ey[i], 0);
-            if (e == cudaSuccess && !fused) e = project_rows(p, p->d_y, r0, r, st);
-            if (e == cudaSuccess) {
+            if (e == cudaSuccess && !fused) e = project_rows(p, p->d_y, r0, r, st, ly);
+            if (e == cudaSuccess && !ly) {
                 qs_launch Li = L;
                 Li.m_base = r0;
                 Li.m_end = r0 + r;
                 e = qs_launch_interp(Li, p->W, p->d_y, fused, st);
             }
         }
+        if (e == cudaSuccess && ly) e = qs_launch_lane_interp(L, p->d_y, from_u, p->d_H, false, st);
         if (e != cudaSuccess) return cuda_fail(e, "qs_sum_host: projection and interpolation of y");
         e = qs_launch_reduce(L, p->d_s, st);
         if (e != cudaSuccess) return cuda_fail(e, "qs_sum_host: reduction");

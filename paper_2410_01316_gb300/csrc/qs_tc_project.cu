@@ -9,7 +9,8 @@
 // shared memory through a ring of stages; one thread issues tcgen05.mma into
 // one of two 256-column FP32 accumulators in tensor memory while eight warps
 // read the other back with tcgen05.ld and store U with one coalesced 128-byte
-// row segment per warp and slice.  tc_project_pair (the default): a cluster
+// row segment per warp and slice, or slice-interleaved (U[p / 32][n][p mod 32],
+// the order that the slice-per-lane grid kernels read) with 32-byte stores.  tc_project_pair (the default): a cluster
 // of two CTAs on an SM pair computes 256-point x 256-slice tiles with
 // cta_group::2 MMAs (M = 256), each CTA holding half of every A and B slab;
 // per SM that cuts the shared-memory traffic of a k-step from 160 to about
@@ -77,6 +78,14 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
         : "memory");
 }
 
@@ -159,6 +168,14 @@ struct TcCfg<1> {  // TF32
     static constexpr uint32_t IDESC = make_idesc(2, TILE_M, TILE_N);
 };
 
+// Back-projection, out = Q Xi: three BF16 parts of either operand, the six products down to 2^-16 of the
+// leading one.  An FP32 number has 24 bits and three parts hold them all.
+template <>
+struct TcCfg<2> {
+    static constexpr int ESZ = 2, BK = 32, NOPS = 3, KSTEP = 16;
+    static constexpr uint32_t IDESC = make_idesc(1, TILE_M, 16);  // 16 columns; the kernel sets the tile's width
+};
+
 constexpr int ROW_BYTES = 64;               // one 64-byte swizzle row per operand row and k-slab
 constexpr int A_BYTES = TILE_M * ROW_BYTES;
 constexpr int B_BYTES = TILE_N * ROW_BYTES;
@@ -192,6 +209,22 @@ template <>
 struct PCfg<1> {  // TF32: 24 KB stages
     static constexpr int STAGES = 8;
 };
+template <>
+struct PCfg<2> {  // back-projection: 72 KB stages
+    static constexpr int STAGES = 3;
+};
+
+// 32 consecutive slices (those of slice group p / 32) of point n, slice-interleaved:
+// U[p / 32][n][32], one full 32-byte sector per store.
+__device__ __forceinline__ void store_lanes(float* __restrict__ U, int64_t ldU, int p, int64_t n, const float (&v)[32])
+{
+    float* o = U + ((size_t)(p >> 5) * ldU + n) * 32;
+#pragma unroll
+    for (int j = 0; j < 32; j += 8)
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o + j), "f"(v[j]), "f"(v[j + 1]),
+                     "f"(v[j + 2]), "f"(v[j + 3]), "f"(v[j + 4]), "f"(v[j + 5]), "f"(v[j + 6]), "f"(v[j + 7])
+                     : "memory");
+}
 
 template <int KIND>
 __host__ __device__ constexpr int tcp_smem_bytes()
@@ -202,11 +235,23 @@ __host__ __device__ constexpr int tcp_smem_bytes()
 constexpr int TCP_EPI_WARPS = 8;  // two per TMEM lane quarter, each storing half the columns
 constexpr int TCP_THREADS = 32 * (2 + TCP_EPI_WARPS);
 
+// What the back-projection (KIND 2) does besides: its inner dimension runs over the slices, 32 of a group
+// per slab (rank-3 maps of the points' parts), its columns are components in tiles of tile_n, and
+// out[n][j] = scale fac_n D[n][j] goes to row-major memory.
+constexpr int BACK_SLABS = 2;  // slabs (64 slices) per accumulator
+struct BackArgs {
+    int tile_n;
+    float scale;
+    const float* fac;
+};
+
 template <int KIND>
 __global__ void __launch_bounds__(TCP_THREADS, 1)
     tc_project_persistent(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
-                          const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1, int d,
-                          int P, int64_t n_base, int64_t N, float* __restrict__ U, int64_t ldU, unsigned int* flag)
+                          const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mB0,
+                          const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mB2, int d,
+                          int P, int64_t n_base, int64_t N, float* __restrict__ U, int64_t ldU, unsigned int* flag,
+                          bool lanes, BackArgs back)
 {
     using C = TcCfg<KIND>;
     constexpr int ST = PCfg<KIND>::STAGES;
@@ -227,7 +272,8 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int nkb = (d + C::BK - 1) / C::BK;
-    const int ptiles = (P + TILE_N - 1) / TILE_N;
+    const int tn = KIND == 2 ? back.tile_n : TILE_N;
+    const int ptiles = (P + tn - 1) / tn;
     const int64_t ntiles = (N + TILE_M - 1) / TILE_M;
     const int64_t T = ntiles * ptiles;
 
@@ -261,7 +307,7 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
         bool ok = true;
         int64_t g = 0;
         for (int64_t t = blockIdx.x; t < T && ok && !abort_all; t += gridDim.x) {
-            const int p0 = (int)(t % ptiles) * TILE_N;
+            const int p0 = (int)(t % ptiles) * tn;
             const int n0 = (int)(n_base + (t / ptiles) * TILE_M);
             for (int kb = 0; kb < nkb; ++kb, ++g) {
                 const int s = (int)(g % ST);
@@ -273,11 +319,18 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
                 const uint32_t fb = full0 + 8 * s;
                 const uint32_t st = tiles + s * SB;
                 const int kc = kb * C::BK;
-                mbar_expect_tx(fb, SB);
-                tma_load_2d(st, &mA0, kc, n0, fb);
-                if (C::NOPS == 2) tma_load_2d(st + A_BYTES, &mA1, kc, n0, fb);
+                mbar_expect_tx(fb, C::NOPS * (A_BYTES + tn * ROW_BYTES));
+                if constexpr (KIND == 2) {
+                    tma_load_3d(st, &mA0, 0, n0, kb, fb);
+                    tma_load_3d(st + A_BYTES, &mA1, 0, n0, kb, fb);
+                    tma_load_3d(st + 2 * A_BYTES, &mA2, 0, n0, kb, fb);
+                    tma_load_2d(st + 3 * A_BYTES + 2 * B_BYTES, &mB2, kc, p0, fb);
+                } else {
+                    tma_load_2d(st, &mA0, kc, n0, fb);
+                    if (C::NOPS == 2) tma_load_2d(st + A_BYTES, &mA1, kc, n0, fb);
+                }
                 tma_load_2d(st + C::NOPS * A_BYTES, &mB0, kc, p0, fb);
-                if (C::NOPS == 2) tma_load_2d(st + C::NOPS * A_BYTES + B_BYTES, &mB1, kc, p0, fb);
+                if (C::NOPS >= 2) tma_load_2d(st + C::NOPS * A_BYTES + B_BYTES, &mB1, kc, p0, fb);
             }
         }
         // no copy of this CTA may still be in flight when it exits
@@ -292,39 +345,53 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
         bool ok = true;
         int64_t g = 0;
         int i = 0;
-        for (int64_t t = blockIdx.x; t < T && ok && !abort_all; t += gridDim.x, ++i) {
-            const int a = i & 1;
-            if (!mbar_wait(tempty0 + 8 * a, (((uint32_t)i >> 1) & 1u) ^ 1u)) {
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t dt = tmem + (uint32_t)(a * TILE_N);
-            for (int kb = 0; kb < nkb; ++kb, ++g) {
-                const int s = (int)(g % ST);
-                if (!mbar_wait(full0 + 8 * s, (uint32_t)(g / ST) & 1u)) {
+        // an accumulator takes a whole tile, or (back-projection) BACK_SLABS slabs of it
+        for (int64_t t = blockIdx.x; t < T && ok && !abort_all; t += gridDim.x) {
+            for (int k0 = 0; k0 < nkb && ok; k0 += KIND == 2 ? BACK_SLABS : nkb, ++i) {
+                const int k1 = KIND == 2 ? min(nkb, k0 + BACK_SLABS) : nkb;
+                const int a = i & 1;
+                if (!mbar_wait(tempty0 + 8 * a, (((uint32_t)i >> 1) & 1u) ^ 1u)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t st = tiles + s * SB;
-                const uint32_t a0 = st, a1 = st + A_BYTES;
-                const uint32_t b0 = st + C::NOPS * A_BYTES, b1 = b0 + B_BYTES;
-#pragma unroll
-                for (int k = 0; k < C::BK / C::KSTEP; ++k) {
-                    const uint32_t off = (uint32_t)(k * C::KSTEP * C::ESZ);
-                    const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u;
-                    if (KIND == 0) {
-                        mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b0 + off), C::IDESC, acc);
-                        mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b1 + off), C::IDESC, 1u);
-                        mma_f16(dt, sw64_desc(a1 + off), sw64_desc(b0 + off), C::IDESC, 1u);
-                    } else {
-                        mma_tf32(dt, sw64_desc(a0 + off), sw64_desc(b0 + off), C::IDESC, acc);
+                const uint32_t dt = tmem + (uint32_t)(a * TILE_N);
+                for (int kb = k0; kb < k1; ++kb, ++g) {
+                    const int s = (int)(g % ST);
+                    if (!mbar_wait(full0 + 8 * s, (uint32_t)(g / ST) & 1u)) {
+                        ok = false;
+                        break;
                     }
+                    tc_fence_after();
+                    const uint32_t st = tiles + s * SB;
+                    const uint32_t a0 = st, a1 = st + A_BYTES;
+                    const uint32_t b0 = st + C::NOPS * A_BYTES, b1 = b0 + B_BYTES;
+#pragma unroll
+                    for (int k = 0; k < C::BK / C::KSTEP; ++k) {
+                        const uint32_t off = (uint32_t)(k * C::KSTEP * C::ESZ);
+                        const uint32_t acc = (kb > k0 || k > 0) ? 1u : 0u;
+                        if constexpr (KIND == 2) {
+                            // the small products first, while the sum they join is small
+                            const uint32_t id = C::IDESC + ((uint32_t)(tn / 8 - 2) << 17), a2 = a1 + A_BYTES,
+                                           b2 = b1 + B_BYTES;
+                            mma_f16(dt, sw64_desc(a2 + off), sw64_desc(b0 + off), id, acc);
+                            mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b2 + off), id, 1u);
+                            mma_f16(dt, sw64_desc(a1 + off), sw64_desc(b1 + off), id, 1u);
+                            mma_f16(dt, sw64_desc(a1 + off), sw64_desc(b0 + off), id, 1u);
+                            mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b1 + off), id, 1u);
+                            mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b0 + off), id, 1u);
+                        } else if (KIND == 0) {
+                            mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b0 + off), C::IDESC, acc);
+                            mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b1 + off), C::IDESC, 1u);
+                            mma_f16(dt, sw64_desc(a1 + off), sw64_desc(b0 + off), C::IDESC, 1u);
+                        } else {
+                            mma_tf32(dt, sw64_desc(a0 + off), sw64_desc(b0 + off), C::IDESC, acc);
+                        }
+                    }
+                    mma_commit(empty0 + 8 * s);
                 }
-                mma_commit(empty0 + 8 * s);
+                if (ok) mma_commit(tfull0 + 8 * a);  // arrives once the accumulator's MMAs have completed
             }
-            if (ok) mma_commit(tfull0 + 8 * a);  // arrives once the tile's MMAs have completed
         }
         // before the tensor memory is freed, every MMA issued above must have finished
         mma_commit(drain);
@@ -341,6 +408,71 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
         int i = 0;
         for (int64_t t = blockIdx.x; t < T; t += gridDim.x, ++i) {
             if (abort_all) break;
+            if constexpr (KIND == 2) {
+                // Each accumulator is added to FP32 sums in registers (32 of the tile's columns at a time, up
+                // to 4 times): the tensor core's own additions truncate, a bias of about 2^-25 of the running
+                // sum each, which 6 P / 16 of them in a row would make 7e-6 of the result (measured, P = 1024).
+                const int half = (tn / 2 + 15) & ~15;
+                const int c0 = h * half, c1 = min(tn, c0 + half);
+                float sum[4][32];
+#pragma unroll
+                for (int q4 = 0; q4 < 4; ++q4)
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) sum[q4][j] = 0.0f;
+                const int chunks = (nkb + BACK_SLABS - 1) / BACK_SLABS;
+                bool got = true;
+                for (int ch = 0; ch < chunks && got; ++ch) {
+                    const int ic = i * chunks + ch, a = ic & 1;
+                    got = __all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * a, ((uint32_t)ic >> 1) & 1u));
+                    if (!got) break;
+                    tc_fence_after();
+                    const uint32_t trow = tmem + (uint32_t)(a * TILE_N) + ((uint32_t)(32 * q) << 16);
+#pragma unroll
+                    for (int q4 = 0; q4 < 4; ++q4) {
+                        if (c0 + 32 * q4 >= c1) continue;
+                        float v[32];
+                        __syncwarp();
+                        tmem_ld32(trow + (uint32_t)(c0 + 32 * q4), v);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) sum[q4][j] += v[j];
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8 * a) : "memory");
+                }
+                if (!got) {
+                    if (lane == 0) {
+                        abort_all = 1;
+                        atomicOr(flag, QS_FLAG_TIMEOUT);
+                    }
+                    break;
+                }
+                const int p0 = (int)(t % ptiles) * tn;
+                const int64_t n = (t / ptiles) * TILE_M + 32 * q + lane;
+                if (n < N) {
+                    const float f = back.scale * (back.fac ? __ldg(&back.fac[n]) : 1.0f);
+                    const bool vec = (ldU & 3) == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
+#pragma unroll
+                    for (int q4 = 0; q4 < 4; ++q4) {
+                        const int pc = p0 + c0 + 32 * q4;
+                        const int cols = min(32, min(P, p0 + c1) - pc);
+                        float* o = U + (size_t)n * ldU + pc;
+                        if (cols == 32 && vec) {
+#pragma unroll
+                            for (int j = 0; j < 32; j += 4)
+                                *reinterpret_cast<float4*>(o + j) = make_float4(sum[q4][j] * f, sum[q4][j + 1] * f,
+                                                                                sum[q4][j + 2] * f, sum[q4][j + 3] * f);
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j)
+                                if (j < cols) o[j] = sum[q4][j] * f;
+                        }
+                    }
+                }
+                __syncwarp();
+                continue;
+            }
             const int a = i & 1;
             const bool got = __all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * a, ((uint32_t)i >> 1) & 1u));
             if (!got) {
@@ -351,7 +483,7 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
                 break;
             }
             tc_fence_after();
-            const int p0 = (int)(t % ptiles) * TILE_N;
+            const int p0 = (int)(t % ptiles) * tn;
             const int64_t n = n_base + (t / ptiles) * TILE_M + 32 * q + lane;
             const uint32_t trow = tmem + (uint32_t)(a * TILE_N) + ((uint32_t)(32 * q) << 16);
 #pragma unroll 1
@@ -360,6 +492,10 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
                 __syncwarp();
                 tmem_ld32(trow + (uint32_t)c, v);
                 const int pc = p0 + c;
+                if (lanes) {
+                    if (pc < P) store_lanes(U, ldU, pc, n, v);  // slices past P: zero directions, zeros
+                    continue;
+                }
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
                     if (pc + j < P) U[(size_t)(pc + j) * ldU + n] = v[j];
@@ -515,7 +651,7 @@ template <int KIND>
 __global__ void __launch_bounds__(TCP_THREADS, 1)
     tc_project_pair(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
                     const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1, int d, int P,
-                    int64_t n_base, int64_t N, float* __restrict__ U, int64_t ldU, unsigned int* flag)
+                    int64_t n_base, int64_t N, float* __restrict__ U, int64_t ldU, unsigned int* flag, bool lanes)
 {
     using C = TcCfg<KIND>;
     constexpr int ST = PairCfg<KIND>::STAGES;
@@ -693,6 +829,10 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
                 __syncwarp();
                 tmem_ld32(trow + (uint32_t)c, v);
                 const int pc = p0 + c;
+                if (lanes) {
+                    if (row_ok && pc < P) store_lanes(U, ldU, pc, n, v);
+                    continue;
+                }
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
                     if (row_ok && pc + j < P) U[(size_t)(pc + j) * ldU + n] = v[j];
@@ -886,7 +1026,7 @@ int pair_clusters()
 
 template <int KIND>
 cudaError_t launch_pair(const CUtensorMap* m, int64_t n_base, int64_t N, int d, int P, float* U, int64_t ldU,
-                        unsigned int* flag, cudaStream_t st)
+                        unsigned int* flag, cudaStream_t st, bool lanes)
 {
     const int ncl_max = pair_clusters<KIND>();
     if (ncl_max <= 0) return cudaErrorNotSupported;
@@ -908,7 +1048,8 @@ cudaError_t launch_pair(const CUtensorMap* m, int64_t n_base, int64_t N, int d, 
     // maps 4 / 5: the directions with 128-row boxes (one CTA's half of a B slab)
     const CUtensorMap& a1 = KIND == 0 ? m[1] : m[0];
     const CUtensorMap& b1 = KIND == 0 ? m[5] : m[4];
-    cudaError_t e = cudaLaunchKernelEx(&cfg, tc_project_pair<KIND>, m[0], a1, m[4], b1, d, P, n_base, N, U, ldU, flag);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, tc_project_pair<KIND>, m[0], a1, m[4], b1, d, P, n_base, N, U, ldU, flag,
+                                       lanes);
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -924,15 +1065,10 @@ int qs_tc_pair_ctas(int kind)
     return 2 * (kind == 0 ? pair_clusters<0>() : pair_clusters<1>());
 }
 
-// maps: [A0, A1, B0, B1, B0 half, B1 half] (A1 / B1 unused by TF32), each a
-// 64-byte-aligned CUtensorMap; B maps 2 / 3 have 256-row boxes, 4 / 5 128-row boxes.
-cudaError_t qs_launch_project_tc(int kind, const void* maps, int64_t n_base, int64_t N, int d, int P, float* U,
-                                 int64_t ldU, unsigned int* flag, cudaStream_t st, bool pair)
+namespace {
+
+cudaError_t sm_count(int* out)
 {
-    if (N <= 0) return cudaSuccess;
-    const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(maps);
-    if (pair) return kind == 0 ? launch_pair<0>(m, n_base, N, d, P, U, ldU, flag, st)
-                               : launch_pair<1>(m, n_base, N, d, P, U, ldU, flag, st);
     static int sms = 0;
     if (!sms) {
         int dev = 0;
@@ -940,6 +1076,95 @@ cudaError_t qs_launch_project_tc(int kind, const void* maps, int64_t n_base, int
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
     }
+    *out = sms;
+    return cudaSuccess;
+}
+
+// Components per tile of the back-projection: d in equal tiles of at most 256, a multiple of 16.
+int back_tile(int d)
+{
+    const int tiles = (d + TILE_N - 1) / TILE_N;
+    return ((d + tiles - 1) / tiles + 15) / 16 * 16;
+}
+
+// xit[part][j][p]: the directions transposed and split into three BF16 parts (zeros past P).
+__global__ void split_xit_kernel(const float* __restrict__ xi, int P, int d, int ldq, __nv_bfloat16* __restrict__ xit)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)d * ldq) return;
+    const int j = (int)(i / ldq), p = (int)(i - (int64_t)j * ldq);
+    float v = p < P ? xi[(size_t)p * d + j] : 0.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const __nv_bfloat16 b = __float2bfloat16_rn(v);
+        xit[(size_t)k * d * ldq + i] = b;
+        v -= __bfloat162float(b);
+    }
+}
+
+}  // namespace
+
+cudaError_t qs_launch_split_xit(const float* xi, int P, int d, int ldq, void* xit, cudaStream_t st)
+{
+    const int64_t n = (int64_t)d * ldq;
+    split_xit_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(xi, P, d, ldq, (__nv_bfloat16*)xit);
+    return cudaGetLastError();
+}
+
+bool qs_make_backproj_maps(unsigned char (*maps)[128], const float* U, const void* qlo, const void* xit, int64_t ldU,
+                           int P, int d, int ldq)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode();
+    if (!enc) return false;
+    // parts of the values: 32 slices of a group (64 bytes) x points x groups; high and middle parts
+    // alternate in U's 128-byte rows
+    const uint16_t* base[3] = {reinterpret_cast<const uint16_t*>(U), reinterpret_cast<const uint16_t*>(U) + 32,
+                               static_cast<const uint16_t*>(qlo)};
+    for (int k = 0; k < 3; ++k) {
+        const cuuint64_t row = k < 2 ? 128 : 64;
+        cuuint64_t gdim[3] = {32, (cuuint64_t)ldU, (cuuint64_t)((P + 31) / 32)};
+        cuuint64_t gstride[2] = {row, row * (cuuint64_t)ldU};
+        cuuint32_t box[3] = {32, TILE_M, 1}, estride[3] = {1, 1, 1};
+        if (enc(reinterpret_cast<CUtensorMap*>(maps[k]), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
+                const_cast<uint16_t*>(base[k]), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+        if (!qs_make_tmap(maps[3 + k], static_cast<const uint16_t*>(xit) + (size_t)k * d * ldq, 2, P, d, ldq, back_tile(d)))
+            return false;
+    }
+    return true;
+}
+
+cudaError_t qs_launch_backproj_tc(const void* maps, int64_t M, int P, int d, float scale, const float* fac, float* out,
+                                  unsigned int* flag, cudaStream_t st)
+{
+    if (M <= 0) return cudaSuccess;
+    const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(maps);
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    const int smem = tcp_smem_bytes<2>(), tn = back_tile(d);
+    e = cudaFuncSetAttribute(tc_project_persistent<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t T = ((M + TILE_M - 1) / TILE_M) * ((d + tn - 1) / tn);
+    tc_project_persistent<2><<<(unsigned)(T < sms ? T : sms), TCP_THREADS, smem, st>>>(
+        m[0], m[1], m[2], m[3], m[4], m[5], P, d, 0, M, out, d, flag, false, BackArgs{tn, scale, fac});
+    return cudaGetLastError();
+}
+
+// maps: [A0, A1, B0, B1, B0 half, B1 half] (A1 / B1 unused by TF32), each a
+// 64-byte-aligned CUtensorMap; B maps 2 / 3 have 256-row boxes, 4 / 5 128-row boxes.
+cudaError_t qs_launch_project_tc(int kind, const void* maps, int64_t n_base, int64_t N, int d, int P, float* U,
+                                 int64_t ldU, unsigned int* flag, cudaStream_t st, bool pair, bool lanes)
+{
+    if (N <= 0) return cudaSuccess;
+    const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(maps);
+    if (pair) return kind == 0 ? launch_pair<0>(m, n_base, N, d, P, U, ldU, flag, st, lanes)
+                               : launch_pair<1>(m, n_base, N, d, P, U, ldU, flag, st, lanes);
+    int sms = 0;
+    cudaError_t es = sm_count(&sms);
+    if (es != cudaSuccess) return es;
     const int64_t T = ((N + TILE_M - 1) / TILE_M) * ((P + TILE_N - 1) / TILE_N);
     const unsigned grid = (unsigned)(T < sms ? T : sms);
     if (kind == 0) {
@@ -947,13 +1172,15 @@ cudaError_t qs_launch_project_tc(int kind, const void* maps, int64_t n_base, int
         cudaError_t e =
             cudaFuncSetAttribute(tc_project_persistent<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        tc_project_persistent<0><<<grid, TCP_THREADS, smem, st>>>(m[0], m[1], m[2], m[3], d, P, n_base, N, U, ldU, flag);
+        tc_project_persistent<0><<<grid, TCP_THREADS, smem, st>>>(m[0], m[1], m[1], m[2], m[3], m[3], d, P, n_base, N, U,
+                                                                  ldU, flag, lanes, BackArgs{});
     } else {
         const int smem = tcp_smem_bytes<1>();
         cudaError_t e =
             cudaFuncSetAttribute(tc_project_persistent<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        tc_project_persistent<1><<<grid, TCP_THREADS, smem, st>>>(m[0], m[0], m[2], m[2], d, P, n_base, N, U, ldU, flag);
+        tc_project_persistent<1><<<grid, TCP_THREADS, smem, st>>>(m[0], m[0], m[0], m[2], m[2], m[2], d, P, n_base, N, U,
+                                                                  ldU, flag, lanes, BackArgs{});
     }
     return cudaGetLastError();
 }
