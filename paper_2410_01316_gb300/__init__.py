@@ -64,9 +64,13 @@ def tune_cache_size() -> int:
 def _stream_handle(stream) -> int:
     import torch
 
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    # the current device's current stream without a Stream object (0.7 against 3.0 us)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is not None:
+        return raw(torch.cuda.current_device())
+    return int(torch.cuda.current_stream().cuda_stream)
 
 
 class QSPlan:

@@ -143,6 +143,41 @@ __global__ void __launch_bounds__(1024) weight_scale_kernel(const float* __restr
     }
 }
 
+// The fixed-point scale and its inverse: from weight_scale_kernel, or, for the
+// few sources of a small problem (QS_INLINE_WEIGHTS), summed by every CTA of
+// the spread itself (the same sum in each): a microsecond of loads and a block
+// reduction there against a launch of 3.5 us ahead of it.  sc: two floats of
+// shared memory; ends with a barrier in the second case.
+__device__ __forceinline__ float2 slice_scale(const qs_launch& L, const float* __restrict__ w, float* sc)
+{
+    if (L.N > QS_INLINE_WEIGHTS) return make_float2(__ldg(&L.wscale[0]), __ldg(&L.wscale[1]));
+    __shared__ float red[32];
+    float acc = 0.0f;
+    if (w)
+        for (int n = threadIdx.x; n < (int)L.N; n += blockDim.x) acc += fabsf(__ldg(&w[n]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float B = 0.0f;
+        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) B += red[i];
+        if (!w) B = (float)L.N;
+        float scale = 0.0f, inv = 0.0f;
+        if (!isfinite(B)) {
+            atomicOr(L.flag, QS_FLAG_NONFINITE);
+        } else if (B > 0.0f) {
+            scale = 1073741824.0f / B;
+            inv = B / 1073741824.0f;
+            if (!isfinite(scale)) scale = inv = 0.0f;  // B below 2^-98: all weights negligible
+        }
+        sc[0] = scale;
+        sc[1] = inv;
+    }
+    __syncthreads();
+    return make_float2(sc[0], sc[1]);
+}
+
 // ---------------------------------------------------------------------------
 // Spread + filter: one CTA per slice p.
 // ---------------------------------------------------------------------------
@@ -262,8 +297,9 @@ __global__ void __launch_bounds__(256) spread_filter_kernel(qs_launch L, const f
         s_lo = INT_MAX;
         s_hi = INT_MIN;
     }
-    const float scale = __ldg(&L.wscale[0]);
-    const float inv_scale = __ldg(&L.wscale[1]);
+    __shared__ float sc[2];
+    const float2 sc2 = slice_scale(L, w, sc);
+    const float scale = sc2.x, inv_scale = sc2.y;
     const float* urow = L.U + (size_t)p * L.ldU;
     __syncthreads();
 
@@ -420,8 +456,9 @@ __device__ __forceinline__ void moment_grid(const qs_launch& L, const float* __r
     const int G = L.G;
     const int cs = G + SPREAD_PAD;
     int* lanewin = tab + cs * KS;
-    const float scale = __ldg(&L.wscale[0]);
-    const float inv_scale = __ldg(&L.wscale[1]);
+    __shared__ float sc[2];
+    const float2 sc2 = slice_scale(L, w, sc);
+    const float scale = sc2.x, inv_scale = sc2.y;
     const float* urow = L.U + (size_t)p * L.ldU;
 
     int wbase = 0;
@@ -625,8 +662,9 @@ __global__ void __launch_bounds__(256) spread_grad_kernel(qs_launch L, const flo
     for (int i = threadIdx.x; i < G + SPREAD_PAD; i += blockDim.x) gridi[i] = 0;
     if (FUSED)
         for (int j = threadIdx.x; j < L.d; j += blockDim.x) xi_sm[j] = L.xi_s[(size_t)p * L.d + j];
-    const float scale = __ldg(&L.wscale[0]);
-    const float inv_scale = __ldg(&L.wscale[1]);
+    __shared__ float sc[2];
+    const float2 sc2 = slice_scale(L, w, sc);
+    const float scale = sc2.x, inv_scale = sc2.y;
     const float* urow = L.U + (size_t)p * L.ldU;
     __syncthreads();
     for (int64_t n = threadIdx.x; n < L.N; n += blockDim.x)
@@ -1230,6 +1268,15 @@ __global__ void __launch_bounds__(256) reduce_grad_kernel(const float* __restric
 // Strips pay while a block per 256 elements leaves SMs idle and a strip still has groups to load.
 bool reduce_in_strips(int S, int64_t n) { return S >= 16 && n <= (int64_t)QS_LANE_CTAS * 256; }
 
+// Opt-in to `smem` bytes of dynamic shared memory, where that and up to 10 KB of static shared memory
+// pass the 48 KB that need none (the call costs about a microsecond of the host's time).
+template <class F>
+cudaError_t opt_in(F kern, size_t smem)
+{
+    if (smem <= 38 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 template <int W, bool FUSED, int MODE, int PARAM, int PF>
 cudaError_t launch_spread_v(const qs_launch& L, const float* x, const float* w, cudaStream_t st)
 {
@@ -1250,7 +1297,7 @@ cudaError_t launch_moment_v(const qs_launch& L, const float* x, const float* w, 
 {
     const size_t smem = qs_moment_smem(L.G, W, LW > 0);
     auto kern = spread_moment_kernel<W, FUSED, LW, 4>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = opt_in(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<L.P, 512, smem, st>>>(L, x, w);
     return cudaGetLastError();
@@ -1286,12 +1333,10 @@ cudaError_t launch_interp_w(const qs_launch& L, const float* y, bool fused, cuda
     if (mt <= 0) return cudaSuccess;
     const unsigned gx = (unsigned)((mt + (int64_t)IT_THREADS * tpt - 1) / ((int64_t)IT_THREADS * tpt));
     dim3 grid(gx, (unsigned)L.S);
-    // the kernel also holds ~8.5 KB of static shared memory, so the opt-in is
-    // needed below 48 KB of dynamic memory too; set it on every launch
 #define QS_LAUNCH_INTERP(FU, DM, TP)                                                                       \
     do {                                                                                                   \
         auto k_ = interp_kernel<W, FU, DM, TP>;                                                            \
-        cudaError_t e_ = cudaFuncSetAttribute(k_, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        cudaError_t e_ = opt_in(k_, smem);                                                                 \
         if (e_ != cudaSuccess) return e_;                                                                  \
         k_<<<grid, IT_THREADS, smem, st>>>(L, y);                                                          \
     } while (0)
@@ -1314,7 +1359,7 @@ cudaError_t launch_spread_grad_w(const qs_launch& L, const float* x, const float
         const size_t smem = (cs * (qs_moment_count(W) + 1) + cs + (mode == 2 ? (size_t)L.G : 0)) * sizeof(float);
         auto kern = mode == 2 ? (fused ? spread_grad_moment_kernel<W, 2, true> : spread_grad_moment_kernel<W, 2, false>)
                               : (fused ? spread_grad_moment_kernel<W, 1, true> : spread_grad_moment_kernel<W, 1, false>);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = opt_in(kern, smem);
         if (e != cudaSuccess) return e;
         kern<<<L.P, 512, smem, st>>>(L, x, w, Dd, H2);
         return cudaGetLastError();
@@ -1451,6 +1496,7 @@ cudaError_t qs_launch_coeffs(int kernel, double kparam, double kparam2, int d, d
 
 cudaError_t qs_launch_weight_scale(const qs_launch& L, const float* w, cudaStream_t st)
 {
+    if (L.N <= QS_INLINE_WEIGHTS) return cudaSuccess;  // the spread's CTAs sum the weights themselves
     weight_scale_kernel<<<1, 1024, 0, st>>>(w, L.N, L.wscale, L.flag);
     return cudaGetLastError();
 }

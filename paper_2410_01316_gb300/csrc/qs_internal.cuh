@@ -34,6 +34,7 @@ constexpr int QS_GRAD_MAX_D = 32;              // largest d of the fused form's 
 constexpr int QS_BATCH_MAX_D = 64;             // largest d of a batched problem
 constexpr int QS_SOBOL_MAX_D = 4096;           // largest d of the Sobol' directions
 constexpr int QS_BATCH_STREAMS = 8;            // streams of a batch's concurrent mode
+constexpr int QS_INLINE_WEIGHTS = 4096;        // most sources whose weights the spread's CTAs sum themselves
 
 // Slice-per-lane grid kernels (qs_lane.cu): the default window width only.
 constexpr int QS_LANE_W = 8;
