@@ -1192,14 +1192,14 @@ __global__ void __launch_bounds__(IT_THREADS) interp_kernel(qs_launch L, const f
     }
 }
 
-// Slice-group partials (part: [hi, lo][S][n]) of element i summed by TwoSum: groups in increasing order
+// Slice-group partials (part: [hi, lo][S][n], without LOW [S][n]) of element i summed by TwoSum: groups in increasing order
 // within each of the block's RS_STRIPS strips of groups, then the strips in order.  Bound by latency for
 // the few elements of small problems: a strip's groups are loaded eight at a time, and the strips side by
 // side make one round of 64 groups' loads out of eight (11.7 -> 4.2 us for 1000 targets, 64 groups; one
 // strip and 256 elements per block where the elements alone fill the SMs).  The result is valid in strip 0.
 constexpr int RS_STRIPS = 8, RS_ELEMS = 32;
 
-template <int STRIPS>
+template <int STRIPS, bool LOW>
 __device__ __forceinline__ void reduce_groups(const float* __restrict__ part, int S, int64_t n, int64_t i, int strip,
                                               float& hi, float& lo)
 {
@@ -1214,7 +1214,7 @@ __device__ __forceinline__ void reduce_groups(const float* __restrict__ part, in
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 a[j] = g + j < g1 ? part[(size_t)(g + j) * n + i] : 0.0f;
-                b[j] = g + j < g1 ? part[(size_t)(S + g + j) * n + i] : 0.0f;
+                b[j] = LOW && g + j < g1 ? part[(size_t)(S + g + j) * n + i] : 0.0f;
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -1239,7 +1239,7 @@ __device__ __forceinline__ void reduce_groups(const float* __restrict__ part, in
 }
 
 // s_m = (1/P) sum over the slice groups.
-template <int STRIPS>
+template <int STRIPS, bool LOW>
 __global__ void __launch_bounds__(256) reduce_kernel(const float* __restrict__ part, int S, int64_t M, int P,
                                                      float* __restrict__ s)
 {
@@ -1247,7 +1247,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(const float* __restrict__ p
     const int64_t m = (int64_t)blockIdx.x * E + threadIdx.x % E;
     const int strip = threadIdx.x / E;
     float hi, lo;
-    reduce_groups<STRIPS>(part, S, M, m, strip, hi, lo);
+    reduce_groups<STRIPS, LOW>(part, S, M, m, strip, hi, lo);
     if (strip == 0 && m < M) s[m] = (hi + lo) / (float)P;
 }
 
@@ -1261,7 +1261,7 @@ __global__ void __launch_bounds__(256) reduce_grad_kernel(const float* __restric
     const int64_t i = (int64_t)blockIdx.x * E + threadIdx.x % E;
     const int strip = threadIdx.x / E;
     float hi, lo;
-    reduce_groups<STRIPS>(part, S, M * d, i, strip, hi, lo);
+    reduce_groups<STRIPS, true>(part, S, M * d, i, strip, hi, lo);
     if (strip == 0 && i < M * d) out[i] = (hi + lo) * scale * (fac ? __ldg(&fac[i / d]) : 1.0f);
 }
 
@@ -1527,9 +1527,10 @@ cudaError_t qs_launch_interp(const qs_launch& L, int W, const float* y, bool fus
 
 cudaError_t qs_launch_reduce(const qs_launch& L, float* s, cudaStream_t st)
 {
-    if (reduce_in_strips(L.S, L.M))
-        reduce_kernel<RS_STRIPS><<<(unsigned)((L.M + RS_ELEMS - 1) / RS_ELEMS), 256, 0, st>>>(L.part, L.S, L.M, L.P, s);
-    else
-        reduce_kernel<1><<<(unsigned)((L.M + 255) / 256), 256, 0, st>>>(L.part, L.S, L.M, L.P, s);
+    const bool strips = reduce_in_strips(L.S, L.M);
+    const unsigned grid = (unsigned)(strips ? (L.M + RS_ELEMS - 1) / RS_ELEMS : (L.M + 255) / 256);
+    auto kern = strips ? (L.lane_part ? reduce_kernel<RS_STRIPS, false> : reduce_kernel<RS_STRIPS, true>)
+                       : (L.lane_part ? reduce_kernel<1, false> : reduce_kernel<1, true>);
+    kern<<<grid, 256, 0, st>>>(L.part, L.S, L.M, L.P, s);
     return cudaGetLastError();
 }

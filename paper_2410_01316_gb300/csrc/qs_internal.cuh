@@ -109,7 +109,7 @@ struct qs_launch {
     float* part;          // 2 x S x M partial slice sums (hi, lo)
     int S;                // number of slice groups of the interpolation
     void* Qlo;            // low BF16 parts of the derivative values (tensor-core forms), [p / 32][m][32]
-    int lane_T;           // targets per CTA of the slice-per-lane interpolation
+    bool lane_part;       // part holds the slice-per-lane interpolation's sums: S x M, no low parts
     unsigned int* flag;   // device error flag
     float* wscale;        // [0] = 2^30 / sum|w| (fixed-point scale of the grids), [1] = its inverse; QS_WSCALE_FLOATS
     int spread_variant;   // QS_SPREAD_* (all variants give bitwise identical grids)
@@ -348,11 +348,11 @@ cudaError_t qs_launch_lane_spread(const qs_launch& L, const float* x, const floa
 // mode 0: plain filter in place; 1: derivative filter in place; 2: plain in place, derivative into H2
 cudaError_t qs_launch_lane_filter(const qs_launch& L, int mode, float* grid, const float* Dd, float* H2,
                                   cudaStream_t st);
-// Slice sums of the rows H into L.part (L.S groups), or (deriv) the values for the back-projection: FP32 into
+// Slice sums of the rows H into L.part (S = qs_lane_groups groups, no low parts), or (deriv) the values for the back-projection: FP32 into
 // L.U, U[p][m]; tensor-core forms as BF16 parts into L.U and L.Qlo.
 cudaError_t qs_launch_lane_interp(const qs_launch& L, const float* y, bool from_u, const float* H, bool deriv,
                                   cudaStream_t st);
-void qs_lane_shape(int64_t M, int P, int S_max, int* T, int* S);
+int qs_lane_groups(int P, int d, bool from_u);
 // Whether the grid stages of n points and P slices run slice-per-lane: the default window, a form whose
 // projections they can take, enough (point, slice) pairs to fill the SMs, and windows that are likely to
 // fit one walk.  The projections of points within R / 2 span G tau R cells, and about 8.4 standard

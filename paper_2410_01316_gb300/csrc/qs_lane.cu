@@ -48,8 +48,15 @@ constexpr int MAGIC_BITS = 0x4B400000;
 // the window's 32 coefficients in registers: as FP32x2 pairs a point's taps
 // are then 12 packed and 8 scalar FMAs, against 32 FMAs each behind a load of
 // its coefficient from the constant bank when they are left there.
-__host__ __device__ constexpr int spread_threads(int D) { return D == 0 ? 768 : (D <= 32 ? 512 : 384); }
-__host__ __device__ constexpr int interp_threads(int D) { return D <= 32 ? 512 : 384; }
+__host__ __device__ constexpr int spread_threads(int D) { return D == 0 ? 768 : (D <= 16 ? 512 : 384); }
+__host__ __device__ constexpr int interp_threads(int D) { return D <= 16 ? 512 : 384; }
+// Slices a lane can hold: two where a point's coordinates are many enough that reading them once for both
+// pays (a 16-byte broadcast takes the shared memory 2 clocks, as many as two taps) and the registers hold
+// both directions.  Their windows have to fit side by side, so it is decided per group of 64 slices, on the
+// spans that the sample finds.  d = 30, 2 x 9.6e5 points, P = 1280: spread 4.02 -> 3.49 ms, interpolation
+// 4.70 -> 3.41 ms; at d = 16 two thirds of the sums are slower with it (windows that only fit singly double
+// the clearing and adding up), at d = 48 the second direction spills (1.55 -> 1.62 ms).
+__host__ __device__ constexpr int lane_slices(int D) { return D == 32 ? 2 : 1; }
 // Each warp stages its points two blocks of SUB at a time: coordinates (row
 // stride D, zeros past d), or projections of the 32 slices (D = 0).
 __host__ __device__ constexpr int lane_stride(int D) { return D > 0 ? D : 32; }
@@ -149,23 +156,29 @@ __device__ __forceinline__ void load_xi(const qs_launch& L, int p, Direction<D>&
     for (int j = 0; j < D; j += 2) xi.c[j / 2] = pack2(at(j), at(j + 1));
 }
 
-// Grid coordinate of the staged point at r on the lane's slice: FP32 products summed in four strands
+// Grid coordinates of the staged point at r on the lane's slices: FP32 products summed in four strands
 // (coordinates mod 4), added at the end.
-template <int D>
-__device__ __forceinline__ float ring_u(const float* r, const Direction<D>& xi, int lane)
+template <int D, int SL>
+__device__ __forceinline__ void ring_u(const float* r, const Direction<D>* xi, int lane, float (&u)[SL])
 {
     if constexpr (D > 0) {
-        f32x2 a = 0, b = 0;
+        f32x2 a[SL], b[SL];
 #pragma unroll
         for (int j = 0; j < D; j += 4) {
             const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(r + j);
-            a = j == 0 ? mul2(xi.c[0], v.x) : fma2(xi.c[j / 2], v.x, a);
-            b = j == 0 ? mul2(xi.c[1], v.y) : fma2(xi.c[j / 2 + 1], v.y, b);
+#pragma unroll
+            for (int h = 0; h < SL; ++h) {
+                a[h] = j == 0 ? mul2(xi[h].c[0], v.x) : fma2(xi[h].c[j / 2], v.x, a[h]);
+                b[h] = j == 0 ? mul2(xi[h].c[1], v.y) : fma2(xi[h].c[j / 2 + 1], v.y, b[h]);
+            }
         }
-        const float2 t = unpack2(add2(a, b));
-        return t.x + t.y;
+#pragma unroll
+        for (int h = 0; h < SL; ++h) {
+            const float2 t = unpack2(add2(a[h], b[h]));
+            u[h] = t.x + t.y;
+        }
     } else {
-        return r[lane];
+        u[0] = r[lane];
     }
 }
 
@@ -220,19 +233,20 @@ __device__ __forceinline__ void taps_of(const Coeffs& k, float s, float (&tap)[W
 __device__ __forceinline__ int lowest_bin(int G) { return -(G >> 1) - (HW - 1); }
 
 // The bins of a sample of the points n0 .. n1 - 1, spaced evenly, into lohi:
-// [0..31] smallest, [32..63] largest of each lane.  scratch: NSAMPLE x D
-// floats (the window itself, not yet in use).  All loads are issued before
-// the first is used: the sample costs one trip to memory.  Ends with a barrier.
-template <int D, int NT>
+// [h][0..31] smallest, [h][32..63] largest of each lane's slice h.  scratch:
+// NSAMPLE x D floats (the window itself, not yet in use).  All loads are issued
+// before the first is used: the sample costs one trip to memory.  Ends with a
+// barrier.
+template <int D, int NT, int SL>
 __device__ __forceinline__ void sample_bins(const qs_launch& L, const float* __restrict__ x, int g, int64_t n0,
-                                            int64_t n1, const Direction<D>& xi, float* scratch, int* lohi)
+                                            int64_t n1, const Direction<D>* xi, float* scratch, int* lohi)
 {
     constexpr int NW = NT / 32, PER = (NSAMPLE + NW - 1) / NW;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ns = (int)min(n1 - n0, (int64_t)NSAMPLE);
-    const int64_t gap = n1 - n0 > NSAMPLE ? (int64_t)((uint64_t)(n1 - n0) / NSAMPLE) : 1;
+    const int64_t gap = n1 - n0 > NSAMPLE ? (int64_t)((uint64_t)(n1 - n0) / NSAMPLE) : 1;  // a shift
     auto at = [&](int i) { return n0 + i * gap; };
-    float u[PER];
+    float us[D > 0 ? 1 : PER];
     if constexpr (D > 0) {
         for (int e = threadIdx.x; e < ns * D; e += blockDim.x) {
             const int i = e / D, j = e % D;
@@ -245,26 +259,53 @@ __device__ __forceinline__ void sample_bins(const qs_launch& L, const float* __r
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             const int i = warp + k * NW;
-            u[k] = i < ns ? __ldcg(&L.U[((size_t)g * L.ldU + at(i)) * 32 + lane]) : 0.0f;
+            us[k] = i < ns ? __ldcg(&L.U[((size_t)g * L.ldU + at(i)) * 32 + lane]) : 0.0f;
         }
     }
-    if (threadIdx.x < 64) lohi[threadIdx.x] = threadIdx.x < 32 ? INT_MAX : INT_MIN;
+    if (threadIdx.x < 64 * SL) lohi[threadIdx.x] = (threadIdx.x & 32) ? INT_MIN : INT_MAX;
     __syncthreads();
-    int lo = INT_MAX, hi = INT_MIN;
+    int lo[SL], hi[SL];
+#pragma unroll
+    for (int h = 0; h < SL; ++h) {
+        lo[h] = INT_MAX;
+        hi[h] = INT_MIN;
+    }
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const int i = warp + k * NW;
         if (i >= ns) break;
-        const float v = D > 0 ? ring_u<D>(scratch + i * D, xi, lane) : u[k];
-        if (!(fabsf(v) <= L.half_G)) continue;
-        float s;
-        const int l0 = (int)(first_cell(v, s) - (unsigned)MAGIC_BITS);
-        lo = min(lo, l0);
-        hi = max(hi, l0);
+        float v[SL];
+        if constexpr (D > 0) ring_u<D, SL>(scratch + i * D, xi, lane, v);
+        else v[0] = us[k];
+#pragma unroll
+        for (int h = 0; h < SL; ++h) {
+            if (!(fabsf(v[h]) <= L.half_G)) continue;
+            float s;
+            const int l0 = (int)(first_cell(v[h], s) - (unsigned)MAGIC_BITS);
+            lo[h] = min(lo[h], l0);
+            hi[h] = max(hi[h], l0);
+        }
     }
-    atomicMin(&lohi[lane], lo);
-    atomicMax(&lohi[32 + lane], hi);
+#pragma unroll
+    for (int h = 0; h < SL; ++h) {
+        atomicMin(&lohi[64 * h + lane], lo[h]);
+        atomicMax(&lohi[64 * h + 32 + lane], hi[h]);
+    }
     __syncthreads();
+}
+
+// A CTA's range of the `total` units of work, `group` in each slice group: an equal share of them all, or
+// (per_group > 0) of one group among per_group CTAs.
+__device__ __forceinline__ void cta_range(int64_t total, int64_t group, int per_group, int64_t& b0, int64_t& b1)
+{
+    if (per_group > 0) {
+        const int g = blockIdx.x / per_group, j = blockIdx.x % per_group;
+        b0 = g * group + j * group / per_group;
+        b1 = g * group + (j + 1) * group / per_group;
+    } else {
+        b0 = (int64_t)blockIdx.x * total / gridDim.x;
+        b1 = (int64_t)(blockIdx.x + 1) * total / gridDim.x;
+    }
 }
 
 // Sampled bins -> the window: its width (bins, the same for all lanes) and the
@@ -275,18 +316,26 @@ struct Window {
     int nb;    // bins of one walk
     int walks;
     bool poly; // polynomials per bin, else cells
-    int base;  // the lane's first bin
 };
 
-// cap_poly / cap_cells: bins that fit as polynomials / as cells.
-__device__ __forceinline__ Window place_window(const int* lohi, int G, int lane, int cap_poly, int cap_cells,
-                                               bool one_walk)
+__device__ __forceinline__ int sampled_need(const int* lohi, int G, int lane)
+{
+    const int lo = lohi[lane], hi = lohi[32 + lane];
+    const int span = lo > hi ? 1 : hi - lo + 1;
+    return min(G, __reduce_max_sync(0xffffffffu, span + 2 * (span >> 2) + 8));
+}
+
+__device__ __forceinline__ int window_base(const int* lohi, int G, int lane, int nbt)
 {
     int lo = lohi[lane], hi = lohi[32 + lane];
     if (lo > hi) lo = hi = 0;
-    const int span = hi - lo + 1;
-    int need = __reduce_max_sync(0xffffffffu, span + 2 * (span >> 2) + 8);
-    need = min(need, G);
+    const int l = lowest_bin(G);
+    return max(l, min(((lo + hi) >> 1) - (nbt >> 1), l + G - nbt));
+}
+
+// cap_poly / cap_cells: bins that fit as polynomials / as cells.
+__device__ __forceinline__ Window place_window(int need, int cap_poly, int cap_cells, bool one_walk)
+{
     Window v;
     v.poly = need <= cap_poly;
     v.walks = 1;
@@ -297,9 +346,14 @@ __device__ __forceinline__ Window place_window(const int* lohi, int G, int lane,
         v.walks = (v.nbt + cap_cells - 1) / cap_cells;
     }
     v.nb = (v.nbt + v.walks - 1) / v.walks;
-    const int l = lowest_bin(G);
-    v.base = max(l, min(((lo + hi) >> 1) - (v.nbt >> 1), l + G - v.nbt));
     return v;
+}
+
+// Two slices per lane where two windows of polynomials fit, or, for spans too wide for one of polynomials,
+// two of cells.
+__device__ __forceinline__ bool pair_windows(int need, int cap_poly, int cap_poly2, int cap_cells2)
+{
+    return need <= cap_poly2 || (need > cap_poly && need <= cap_cells2);
 }
 
 // ---------------------------------------------------------------------------
@@ -485,16 +539,19 @@ __device__ __forceinline__ unsigned spread_one(float u, float ws, unsigned first
     return rel;
 }
 
-// The points n0 .. n0 + cnt - 1 into the window of one walk.
-template <int D, bool POLY, bool FAST>
+// The points n0 .. n0 + cnt - 1 into the windows of one walk, `cols` and `wstride` ints apart.
+template <int D, int SL, bool POLY, bool FAST>
 __device__ __forceinline__ void spread_walk(const qs_launch& L, const float* __restrict__ x,
-                                            const float* __restrict__ w, float wscale, float scale, int g, int64_t n0, int cnt,
-                                            const Direction<D>& xi, float* ring, int* col, const Window& v, int walk,
-                                            int* row, const f32x2* coef)
+                                            const float* __restrict__ w, float wscale, float scale, int g, int64_t n0,
+                                            int cnt, const Direction<D>* xi, float* ring, int* cols, int wstride,
+                                            const Window& v, const int (&base)[SL], int walk, int* Hi, int p,
+                                            const f32x2* coef)
 {
     constexpr int RS = lane_stride(D), STEP = spread_threads(D) / 32 * SUB;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned first0 = (unsigned)(MAGIC_BITS + v.base), first = first0 + (unsigned)(walk * v.nb);
+    unsigned first[SL];
+#pragma unroll
+    for (int h = 0; h < SL; ++h) first[h] = (unsigned)(MAGIC_BITS + base[h] + walk * v.nb);
     const unsigned nb = (unsigned)min(v.nb, v.nbt - walk * v.nb);
     const unsigned dump = POLY ? nb : nb + (W - 1);
     Coeffs cf;
@@ -524,16 +581,24 @@ __device__ __forceinline__ void spread_walk(const qs_launch& L, const float* __r
         const float* r = ring + buf;
         unsigned worst = 0;
 #pragma unroll
-        for (int i = 0; i < SUB; ++i)
-            worst = max(worst, spread_one<POLY, FAST>(ring_u<D>(r + i * RS, xi, lane), __shfl_sync(0xffffffffu, wk, i),
-                                                      first, nb, dump, col, cf));
+        for (int i = 0; i < SUB; ++i) {
+            float u[SL];
+            ring_u<D, SL>(r + i * RS, xi, lane, u);
+            const float ws = __shfl_sync(0xffffffffu, wk, i);
+#pragma unroll
+            for (int h = 0; h < SL; ++h)
+                worst = max(worst, spread_one<POLY, FAST>(u[h], ws, first[h], nb, dump, cols + h * wstride, cf));
+        }
         if (worst >= nb && walk == 0) {
             // points past the last have weight 0 and whatever the ring held: not looked at
             for (int i = 0; i < SUB && b + i < cnt; ++i) {
-                float s;
-                const float u = ring_u<D>(r + i * RS, xi, lane);
-                if (first_cell(u, s) - first0 >= (unsigned)v.nbt)
-                    spread_outside(L, u, (wsrc ? __ldg(&wsrc[b + i]) : 1.0f) * scale, row);
+                float u[SL], s;
+                ring_u<D, SL>(r + i * RS, xi, lane, u);
+#pragma unroll
+                for (int h = 0; h < SL; ++h)
+                    if (first_cell(u[h], s) - (unsigned)(MAGIC_BITS + base[h]) >= (unsigned)v.nbt)
+                        spread_outside(L, u[h], (wsrc ? __ldg(&wsrc[b + i]) : 1.0f) * scale,
+                                       Hi + (size_t)min(p + 32 * h, L.P - 1) * L.G);
             }
         }
         __syncwarp();  // this stage is refilled by the next step
@@ -620,68 +685,121 @@ __device__ __forceinline__ void add_moments(const qs_launch& L, const int* col, 
     }
 }
 
+// Everything about one CTA's share of a group's points that does not depend on the group.
+struct SpreadShare {
+    const float* x;
+    const float* w;
+    int* Hi;
+    int* win;
+    float* ring;
+    float* red;
+    const f32x2* coef;
+    float scale, wmax;
+};
+
+// The points n0 .. n1 - 1 onto SL slices per lane, the first at p.
+template <int D, int SL>
+__device__ __forceinline__ void spread_slices(const qs_launch& L, const SpreadShare& c, int g, int p, int64_t n0,
+                                              int64_t n1, const Direction<D>* xi, const Window& v,
+                                              const int (&base)[SL])
+{
+    const int lane = threadIdx.x & 31;
+    int* col = c.win + lane;
+    const int64_t most = v.poly ? n1 - n0 : (int64_t)CELL_POINTS;
+    for (int64_t m0 = n0; m0 < n1; m0 += most) {
+        const int cnt = (int)min(most, n1 - m0);
+        const int finer = finer_bits(c.w, m0, m0 + cnt, c.scale, c.red);
+        const float ws = c.scale * (float)(1 << finer);
+        const bool fast = c.wmax * (float)(1 << finer) < 2097152.0f;
+        for (int walk = 0; walk < v.walks; ++walk) {
+            const int nb = min(v.nb, v.nbt - walk * v.nb);
+            // per slice: the window, and behind it the bin that nobody reads
+            const int rows = v.poly ? nb * K : nb + W - 1, stride = (v.poly ? (nb + 1) * K : nb + 2 * W - 1) * 32;
+            __syncthreads();
+#pragma unroll
+            for (int h = 0; h < SL; ++h)
+                for (int i = threadIdx.x; i < rows * 8; i += blockDim.x)
+                    reinterpret_cast<int4*>(c.win + h * stride)[i] = make_int4(0, 0, 0, 0);
+            __syncthreads();
+            if (v.poly) {
+                if (fast) spread_walk<D, SL, true, true>(L, c.x, c.w, ws, c.scale, g, m0, cnt, xi, c.ring, col, stride, v, base, walk, c.Hi, p, c.coef);
+                else spread_walk<D, SL, true, false>(L, c.x, c.w, ws, c.scale, g, m0, cnt, xi, c.ring, col, stride, v, base, walk, c.Hi, p, c.coef);
+            } else {
+                if (fast) spread_walk<D, SL, false, true>(L, c.x, c.w, ws, c.scale, g, m0, cnt, xi, c.ring, col, stride, v, base, walk, c.Hi, p, c.coef);
+                else spread_walk<D, SL, false, false>(L, c.x, c.w, ws, c.scale, g, m0, cnt, xi, c.ring, col, stride, v, base, walk, c.Hi, p, c.coef);
+            }
+            __syncthreads();
+#pragma unroll 1
+            for (int h = 0; h < SL; ++h) {
+                const int at = (SL > 1 && h ? base[SL - 1] : base[0]) + walk * v.nb, ph = p + 32 * h;
+                if (v.poly) add_moments<D>(L, col + h * stride, nb, at, finer, ph < L.P ? c.Hi + (size_t)ph * L.G : nullptr);
+                else add_cells(c.win + h * stride, nb + W - 1, at, finer, ph - lane, L.P, L.G, c.Hi);
+            }
+        }
+    }
+    __syncthreads();
+}
+
 template <int D>
 __global__ void __launch_bounds__(spread_threads(D), 1)
     lane_spread_kernel(const __grid_constant__ qs_launch L, const float* __restrict__ x, const float* __restrict__ w,
-                       int* __restrict__ Hi, int win_bytes)
+                       int* __restrict__ Hi, int win_bytes, int per_group)
 {
+    constexpr int SL = lane_slices(D);
     extern __shared__ float4 smem4[];
-    int* win = reinterpret_cast<int*>(smem4);
-    __shared__ int lohi[64];
+    __shared__ int lohi[64 * SL];
     __shared__ f32x2 coef[HW * T4];
+    __shared__ float red[32];
     share_coeffs(L.win, coef);  // read after the first barrier
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int G = L.G;
     if (__ldg(&L.wscale[3]) != 0.0f) return;  // non-finite weights: flagged, the grids stay zero
-    const float scale = __ldg(&L.wscale[0]);
-    const float wmax = __ldg(&L.wscale[2]);
-    __shared__ float red[32];
-    float* ring = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(smem4) + win_bytes) +
-                  warp * lane_ring_floats(D);
-    for (int i = lane; i < lane_ring_floats(D); i += 32) ring[i] = 0.0f;
+    SpreadShare c;
+    c.x = x;
+    c.w = w;
+    c.Hi = Hi;
+    c.win = reinterpret_cast<int*>(smem4);
+    c.ring = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(smem4) + win_bytes) + warp * lane_ring_floats(D);
+    c.red = red;
+    c.coef = coef;
+    c.scale = __ldg(&L.wscale[0]);
+    c.wmax = __ldg(&L.wscale[2]);
+    for (int i = lane; i < lane_ring_floats(D); i += 32) c.ring[i] = 0.0f;
 
+    const int cap_poly = win_bytes / (K * 128) - 1, cap_cells = win_bytes / 128 - (2 * W - 1);
     const int64_t nsb = (L.N + SUB - 1) / SUB;
-    const int64_t total = nsb * ((L.P + 31) / 32);
-    const int64_t b0 = (int64_t)blockIdx.x * total / gridDim.x, b1 = (int64_t)(blockIdx.x + 1) * total / gridDim.x;
-    for (int64_t b = b0; b < b1;) {
+    int64_t b, b1;
+    cta_range(nsb * ((L.P + 32 * SL - 1) / (32 * SL)), nsb, per_group, b, b1);
+    while (b < b1) {
         const int g = (int)(b / nsb);
         const int64_t e = min(b1, (int64_t)(g + 1) * nsb);
         const int64_t n0 = (b - (int64_t)g * nsb) * SUB, n1 = min(L.N, (e - (int64_t)g * nsb) * SUB);
         b = e;
-        const int p = 32 * g + lane;
-        Direction<D> xi;
-        load_xi<D>(L, p, xi);
-        sample_bins<D, spread_threads(D)>(L, x, g, 0, L.N, xi, reinterpret_cast<float*>(win), lohi);
-        const Window v = place_window(lohi, G, lane, win_bytes / (K * 128) - 1, win_bytes / 128 - (2 * W - 1), false);
-        int* col = win + lane;
-        int* row = Hi + (size_t)min(p, L.P - 1) * G;
-        const int64_t most = v.poly ? n1 - n0 : (int64_t)CELL_POINTS;
-        for (int64_t c = n0; c < n1; c += most) {
-            const int cnt = (int)min(most, n1 - c);
-            const int finer = finer_bits(w, c, c + cnt, scale, red);
-            const float wscale = scale * (float)(1 << finer);
-            const bool fast = wmax * (float)(1 << finer) < 2097152.0f;
-            for (int walk = 0; walk < v.walks; ++walk) {
-                const int nb = min(v.nb, v.nbt - walk * v.nb);
-                const int rows = v.poly ? nb * K : nb + W - 1;
-                __syncthreads();
-                for (int i = threadIdx.x; i < rows * 8; i += blockDim.x)
-                    reinterpret_cast<int4*>(win)[i] = make_int4(0, 0, 0, 0);
-                __syncthreads();
-                if (v.poly) {
-                    if (fast) spread_walk<D, true, true>(L, x, w, wscale, scale, g, c, cnt, xi, ring, col, v, walk, row, coef);
-                    else spread_walk<D, true, false>(L, x, w, wscale, scale, g, c, cnt, xi, ring, col, v, walk, row, coef);
-                } else {
-                    if (fast) spread_walk<D, false, true>(L, x, w, wscale, scale, g, c, cnt, xi, ring, col, v, walk, row, coef);
-                    else spread_walk<D, false, false>(L, x, w, wscale, scale, g, c, cnt, xi, ring, col, v, walk, row, coef);
-                }
-                __syncthreads();
-                const int at = v.base + walk * v.nb;
-                if (v.poly) add_moments<D>(L, col, nb, at, finer, p < L.P ? row : nullptr);
-                else add_cells(win, nb + W - 1, at, finer, 32 * g, L.P, G, Hi);
+        const int p = 32 * SL * g + lane;
+        Direction<D> xi[SL];
+#pragma unroll
+        for (int h = 0; h < SL; ++h) load_xi<D>(L, p + 32 * h, xi[h]);
+        sample_bins<D, spread_threads(D), SL>(L, x, g, 0, L.N, xi, reinterpret_cast<float*>(c.win), lohi);
+        int need[SL];
+#pragma unroll
+        for (int h = 0; h < SL; ++h) need[h] = sampled_need(lohi + 64 * h, G, lane);
+        if constexpr (SL == 2) {
+            const int most = max(need[0], need[1]);
+            const int cap_poly2 = win_bytes / 2 / (K * 128) - 1, cap_cells2 = win_bytes / 2 / 128 - (2 * W - 1);
+            if (p - lane + 32 < L.P && pair_windows(most, cap_poly, cap_poly2, cap_cells2)) {
+                const Window v = place_window(most, cap_poly2, cap_cells2, false);
+                const int base[2] = {window_base(lohi, G, lane, v.nbt), window_base(lohi + 64, G, lane, v.nbt)};
+                spread_slices<D, 2>(L, c, g, p, n0, n1, xi, v, base);
+                continue;
             }
         }
-        __syncthreads();
+#pragma unroll 1
+        for (int h = 0; h < SL && p - lane + 32 * h < L.P; ++h) {
+            if (h) load_xi<D>(L, p + 32 * h, xi[0]);
+            const Window v = place_window(h ? need[SL - 1] : need[0], cap_poly, cap_cells, false);
+            const int base[1] = {window_base(lohi + 64 * h, G, lane, v.nbt)};
+            spread_slices<D, 1>(L, c, g, p + 32 * h, n0, n1, xi, v, base);
+        }
     }
 }
 
@@ -723,13 +841,16 @@ __global__ void __launch_bounds__(256) lane_filter_kernel(const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------
-// Interpolation.  CTA (chunk of L.lane_T targets, slice groups [s NG / S,
-// (s + 1) NG / S)); per group it stages the windows of the 32 filtered rows
-// and its warps walk over the targets, 32 slices at a time.  The 32 values of
-// a target are added across the lanes as the targets go by -- pairs of targets
-// over lane bit 0, pairs of pairs over bit 1, and so on, one shuffle per
-// target in all -- after which lane l holds the group's sum of target l of the
-// block; the groups' sums are accumulated by TwoSum in increasing order.
+// Interpolation.  The (slice group, block of 32 targets) pairs are cut into one
+// contiguous range per CTA like the spread's: a CTA stages the windows of the
+// filtered rows once or twice, and every SM gets the same number of targets.
+// (A grid of target chunks x group ranges left 39 % of the SM time idle at
+// 2e4 targets and 32 groups, and staged a window per group and chunk.)  The 32
+// values of a target are added across the lanes as the targets go by -- pairs
+// of targets over lane bit 0, pairs of pairs over bit 1, and so on, one shuffle
+// per target in all -- after which lane l holds the group's sum of target l of
+// the block, written to part[g][m]; the groups' sums are accumulated by TwoSum
+// in increasing order by the reduction.
 // ---------------------------------------------------------------------------
 template <int B>
 __device__ __forceinline__ float fold(float a, float b, int lane)
@@ -779,16 +900,19 @@ __device__ __forceinline__ float interp_one(float u, unsigned first, unsigned nb
     return v;
 }
 
-// The targets m0 .. m0 + cnt - 1 against the window of one walk: blocks of 32
+// The targets m0 .. m0 + cnt - 1 against the windows of one walk: blocks of 32
 // targets per warp, in steps of SUB.
-template <int D, int OUT, bool POLY>
+template <int D, int SL, int OUT, bool POLY>
 __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __restrict__ y, int g, int64_t m0,
-                                            int cnt, const Direction<D>& xi, float* ring, const float* col,
-                                            const Window& v, int walk, const float* row, float* acc, const f32x2* coef)
+                                            int cnt, const Direction<D>* xi, float* ring, const float* cols,
+                                            int wstride, const Window& v, const int (&base)[SL], int walk,
+                                            const float* H, int p, bool more, const f32x2* coef)
 {
     constexpr int RS = lane_stride(D), NW = interp_threads(D) / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned first0 = (unsigned)(MAGIC_BITS + v.base), first = first0 + (unsigned)(walk * v.nb);
+    unsigned first[SL];
+#pragma unroll
+    for (int h = 0; h < SL; ++h) first[h] = (unsigned)(MAGIC_BITS + base[h] + walk * v.nb);
     const unsigned nb = (unsigned)min(v.nb, v.nbt - walk * v.nb);
     const unsigned dump = POLY ? nb : nb + (W - 1);
     Coeffs cf;
@@ -808,24 +932,24 @@ __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __r
     // OUT = 1, a value for the back-projection.  Unfused FP32: U[p][m].  Tensor-core forms: as three BF16
     // parts, high and middle in place of the projection (64 bytes each of the 128 of target m's 32
     // slices), low in Qlo, K-major operands of the back-projection GEMM.
-    const int p = 32 * g + lane;
-    auto put = [&](int m, float q, bool ok) {
+    auto put = [&](int h, int m, float q, bool ok) {
         if (!ok || m >= cnt) return;
         if constexpr (D > 0) {
-            if (p < L.P) L.U[(size_t)p * L.ldU + m0 + m] = q;
+            if (p + 32 * h < L.P) L.U[(size_t)(p + 32 * h) * L.ldU + m0 + m] = q;
         } else {
             __nv_bfloat16* hm = reinterpret_cast<__nv_bfloat16*>(U + (size_t)m * 32);
-            const __nv_bfloat16 h = __float2bfloat16_rn(q);
-            const float q1 = q - __bfloat162float(h);
+            const __nv_bfloat16 hi = __float2bfloat16_rn(q);
+            const float q1 = q - __bfloat162float(hi);
             const __nv_bfloat16 md = __float2bfloat16_rn(q1);
-            hm[lane] = h;
+            hm[lane] = hi;
             hm[32 + lane] = md;
             reinterpret_cast<__nv_bfloat16*>(L.Qlo)[((size_t)g * L.ldU + m0 + m) * 32 + lane] =
                 __float2bfloat16_rn(q1 - __bfloat162float(md));
         }
     };
+    float* part = L.part + (size_t)g * L.M + m0;
     fetch(warp * 32, 0);
-    float f3 = 0.0f, f4 = 0.0f;
+    float f3 = 0.0f, f4 = 0.0f, far = 0.0f;
     int buf = 0;
     for (int b = warp * 32; b < ((cnt + 31) & ~31); buf ^= SUB * RS) {
         const int next = (b & 24) == 24 ? b - 24 + NW * 32 : b + SUB;
@@ -833,55 +957,65 @@ __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __r
         cp_async_wait<1>();
         __syncwarp();
         const float* r = ring + buf;
-        float f[2], all[OUT == 1 && D > 0 ? SUB : 1];
+        float f[2], all[OUT == 1 && D > 0 ? SL : 1][OUT == 1 && D > 0 ? SUB : 1];
         unsigned worst = 0;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int q = 0; q < 2; ++q) {
             float val[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const int j = 4 * h + i;
-                unsigned rel;
-                val[i] = interp_one<POLY>(ring_u<D>(r + j * RS, xi, lane), first, nb, dump, col, cf, rel);
-                worst = max(worst, rel);
-                if constexpr (OUT == 1 && D > 0) all[j] = val[i];
-                else if (OUT == 1) put(b + j, val[i], rel < nb);
+                const int j = 4 * q + i;
+                float u[SL];
+                ring_u<D, SL>(r + j * RS, xi, lane, u);
+                val[i] = 0.0f;
+#pragma unroll
+                for (int h = 0; h < SL; ++h) {
+                    unsigned rel;
+                    const float t = interp_one<POLY>(u[h], first[h], nb, dump, cols + h * wstride, cf, rel);
+                    worst = max(worst, rel);
+                    val[i] = h ? val[i] + t : t;
+                    if constexpr (OUT == 1 && D > 0) all[h][j] = t;
+                    else if (OUT == 1) put(h, b + j, t, rel < nb);
+                }
             }
-            if (OUT == 0) f[h] = fold<1>(fold<0>(val[0], val[1], lane), fold<0>(val[2], val[3], lane), lane);
+            if (OUT == 0) f[q] = fold<1>(fold<0>(val[0], val[1], lane), fold<0>(val[2], val[3], lane), lane);
         }
         if constexpr (OUT == 1 && D > 0) {
             // eight consecutive values of the lane's slice: one 32-byte sector (U's rows are padded to 128)
             if (worst < nb) {
-                if (p < L.P) {
-                    float4* o = reinterpret_cast<float4*>(L.U + (size_t)p * L.ldU + m0 + b);
-                    o[0] = make_float4(all[0], all[1], all[2], all[3]);
-                    o[1] = make_float4(all[4], all[5], all[6], all[7]);
-                }
+#pragma unroll
+                for (int h = 0; h < SL; ++h)
+                    if (p + 32 * h < L.P) {
+                        float4* o = reinterpret_cast<float4*>(L.U + (size_t)(p + 32 * h) * L.ldU + m0 + b);
+                        o[0] = make_float4(all[h][0], all[h][1], all[h][2], all[h][3]);
+                        o[1] = make_float4(all[h][4], all[h][5], all[h][6], all[h][7]);
+                    }
             } else {
 #pragma unroll
                 for (int i = 0; i < SUB; ++i) {
-                    float s;
-                    put(b + i, all[i], first_cell(ring_u<D>(r + i * RS, xi, lane), s) - first < nb);
+                    float u[SL], s;
+                    ring_u<D, SL>(r + i * RS, xi, lane, u);
+#pragma unroll
+                    for (int h = 0; h < SL; ++h) put(h, b + i, all[h][i], first_cell(u[h], s) - first[h] < nb);
                 }
             }
         }
         if (walk == 0 && __any_sync(0xffffffffu, worst >= nb)) {
             for (int i = 0; i < SUB && b + i < cnt; ++i) {
-                float s, t = 0.0f;
-                const float u = ring_u<D>(r + i * RS, xi, lane);
-                if (first_cell(u, s) - first0 >= (unsigned)v.nbt) {
-                    t = interp_outside(L, u, row);
-                    if (OUT == 1) put(b + i, t, true);
-                }
+                float u[SL], s, t = 0.0f;
+                ring_u<D, SL>(r + i * RS, xi, lane, u);
+#pragma unroll
+                for (int h = 0; h < SL; ++h)
+                    if (first_cell(u[h], s) - (unsigned)(MAGIC_BITS + base[h]) >= (unsigned)v.nbt) {
+                        const int ph = p + 32 * h;
+                        const float q = interp_outside(L, u[h], H + (size_t)min(ph, L.P - 1) * L.G);
+                        if (OUT == 1) put(h, b + i, q, true);
+                        t += q;
+                    }
                 if (OUT == 0) {
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                    if (lane == 0) {
-                        float hi = acc[b + i], lo = acc[L.lane_T + b + i];
-                        qs_two_sum(hi, lo, t);
-                        acc[b + i] = hi;
-                        acc[L.lane_T + b + i] = lo;
-                    }
+                    if (lane == ((b + i) & 31)) far = t;
                 }
             }
             __syncwarp();
@@ -895,12 +1029,11 @@ __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __r
                 if ((b & 16) == 0) {
                     f4 = t;
                 } else {
-                    t = fold<4>(f4, t, lane);
+                    t = fold<4>(f4, t, lane) + far;
+                    far = 0.0f;
                     const int at = (b & ~31) + lane;
-                    float hi = acc[at], lo = acc[L.lane_T + at];
-                    qs_two_sum(hi, lo, t);
-                    acc[at] = hi;
-                    acc[L.lane_T + at] = lo;
+                    // `more`: the group's other slices, or another walk's targets, came before
+                    if (at < cnt) part[at] = more ? part[at] + t : t;
                 }
             }
         }
@@ -910,96 +1043,147 @@ __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __r
     cp_async_wait<0>();
 }
 
-template <int D, int OUT>
-__global__ void __launch_bounds__(interp_threads(D), 1)
-    lane_interp_kernel(const __grid_constant__ qs_launch L, const float* __restrict__ y, const float* __restrict__ H,
-                       int win_bytes)
+// Bins that fit into `bytes` as polynomials (with the cells that they are formed from: n + W - 1, up to 3
+// of alignment, and the zeros that points outside read) and as cells.
+__device__ __forceinline__ int interp_cap_poly(int bytes) { return (bytes / 128 - (K + W)) / (K + 1); }
+__device__ __forceinline__ int interp_cap_cells(int bytes) { return bytes / 128 - 2 * W; }
+
+// The window of walk `walk` of the lane's row into win (`stride` rows of 32 in all); a barrier is the caller's.
+template <int NT>
+__device__ __forceinline__ void stage_cells(const qs_launch& L, const float* row, bool live, int b0, int nb, bool poly,
+                                            float* win)
 {
-    extern __shared__ float4 smem4[];
-    unsigned char* sm = reinterpret_cast<unsigned char*>(smem4);
-    float* win = reinterpret_cast<float*>(smem4);
-    float* acc = reinterpret_cast<float*>(sm + win_bytes + lane_ring_bytes(D, interp_threads(D)));
-    __shared__ int lohi[64];
-    __shared__ f32x2 coef[HW * T4];
-    share_coeffs(L.win, coef);  // read after the first barrier
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    float* ring = reinterpret_cast<float*>(sm + win_bytes) + warp * lane_ring_floats(D);
-    for (int i = lane; i < lane_ring_floats(D); i += 32) ring[i] = 0.0f;
-    const int G = L.G, mask = G - 1;
-    const int chunk = blockIdx.x / L.S, s = blockIdx.x % L.S;
-    const int NG = (L.P + 31) / 32;
-    const int g0 = (int)((int64_t)s * NG / L.S), g1 = (int)((int64_t)(s + 1) * NG / L.S);
-    const int64_t m0 = L.m_base + (int64_t)chunk * L.lane_T, m1 = min(L.m_end, m0 + L.lane_T);
-    if (OUT == 0)
-        for (int i = threadIdx.x; i < 2 * L.lane_T; i += blockDim.x) acc[i] = 0.0f;
-    for (int g = g0; g < g1; ++g) {
-        const int p = 32 * g + lane;
-        Direction<D> xi;
-        load_xi<D>(L, p, xi);
-        __syncthreads();  // the last group's window is done with
-        sample_bins<D, interp_threads(D)>(L, y, g, m0, m1, xi, win, lohi);
-        // polynomials of n bins also need their n + W - 1 cells (and up to 3 of alignment) while they
-        // are formed; values written over their own projections allow one walk only
-        const Window v = place_window(lohi, G, lane, (win_bytes / 128 - (K + W)) / (K + 1), win_bytes / 128 - 2 * W,
-                                      OUT == 1 && D == 0);
-        const float* row = H + (size_t)min(p, L.P - 1) * G;
-        for (int walk = 0; walk < v.walks; ++walk) {
-            const int nb = min(v.nb, v.nbt - walk * v.nb);
-            const int b0 = v.base + walk * v.nb;
-            // the cells b0 & ~3 .. of each lane's row, four at a time (rows are 16-byte aligned, G a multiple of 4)
-            const int a0 = b0 & ~3, off = b0 - a0;
-            const int n4 = (nb + W - 1 + 3 + 3) >> 2;
-            // behind the window: the zeros that points outside read
-            float* cells = v.poly ? win + (nb + 1) * K * 32 : win;
-            float* zeros = win + (v.poly ? nb * K : nb + W - 1) * 32;
-            __syncthreads();
-            for (int c0 = warp; c0 < n4; c0 += 4 * nw) {
-                float4 t[4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, mask = L.G - 1;
+    constexpr int nw = NT / 32;
+    // the cells b0 & ~3 .. of each lane's row, four at a time (rows are 16-byte aligned, G a multiple of 4)
+    const int a0 = b0 & ~3, off = b0 - a0;
+    const int n4 = (nb + W - 1 + 3 + 3) >> 2;
+    // behind the window: the zeros that points outside read
+    float* cells = poly ? win + (nb + 1) * K * 32 : win;
+    float* zeros = win + (poly ? nb * K : nb + W - 1) * 32;
+    for (int c0 = warp; c0 < n4; c0 += 4 * nw) {
+        float4 t[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int c = c0 + k * nw;
-                    t[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                    if (c < n4 && p < L.P) t[k] = __ldcg(reinterpret_cast<const float4*>(row + ((a0 + 4 * c) & mask)));
-                }
+        for (int k = 0; k < 4; ++k) {
+            const int c = c0 + k * nw;
+            t[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (c < n4 && live) t[k] = __ldcg(reinterpret_cast<const float4*>(row + ((a0 + 4 * c) & mask)));
+        }
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    // lanes with another alignment shift their cells; those before the first or after
-                    // the last bin's are dropped
-                    const float e[4] = {t[k].x, t[k].y, t[k].z, t[k].w};
+        for (int k = 0; k < 4; ++k) {
+            // lanes with another alignment shift their cells; those before the first or after
+            // the last bin's are dropped
+            const float e[4] = {t[k].x, t[k].y, t[k].z, t[k].w};
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int r = 4 * (c0 + k * nw) + i - off;
-                        if (r >= 0 && r < nb + W - 1) cells[r * 32 + lane] = e[i];
-                    }
-                }
-            }
-            for (int i = threadIdx.x; i < K * 32; i += blockDim.x) zeros[i] = 0.0f;
-            __syncthreads();
-            if (v.poly) {
-                for (int b = warp; b < nb; b += nw) {
-                    float r[W];
-#pragma unroll
-                    for (int j = 0; j < W; ++j) r[j] = cells[(b + j) * 32 + lane];
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        float q = 0.0f;
-#pragma unroll
-                        for (int j = 0; j < W; ++j) q = fmaf(L.atab[j * K + k], r[j], q);
-                        win[(b * K + k) * 32 + lane] = q;
-                    }
-                }
-                __syncthreads();
-                interp_walk<D, OUT, true>(L, y, g, m0, (int)(m1 - m0), xi, ring, win + lane, v, walk, row, acc, coef);
-            } else {
-                interp_walk<D, OUT, false>(L, y, g, m0, (int)(m1 - m0), xi, ring, win + lane, v, walk, row, acc, coef);
+            for (int i = 0; i < 4; ++i) {
+                const int r = 4 * (c0 + k * nw) + i - off;
+                if (r >= 0 && r < nb + W - 1) cells[r * 32 + lane] = e[i];
             }
         }
     }
-    if (OUT == 0) {
+    for (int i = threadIdx.x; i < K * 32; i += blockDim.x) zeros[i] = 0.0f;
+}
+
+// The bins' polynomials from the staged cells.
+template <int NT>
+__device__ __forceinline__ void form_polynomials(const qs_launch& L, int nb, float* win)
+{
+    const int lane = threadIdx.x & 31;
+    const float* cells = win + (nb + 1) * K * 32;
+    for (int b = threadIdx.x >> 5; b < nb; b += NT / 32) {
+        float r[W];
+#pragma unroll
+        for (int j = 0; j < W; ++j) r[j] = cells[(b + j) * 32 + lane];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            float q = 0.0f;
+#pragma unroll
+            for (int j = 0; j < W; ++j) q = fmaf(L.atab[j * K + k], r[j], q);
+            win[(b * K + k) * 32 + lane] = q;
+        }
+    }
+}
+
+// The CTA's targets against SL slices per lane, the first at p.
+template <int D, int SL, int OUT>
+__device__ __forceinline__ void interp_slices(const qs_launch& L, const float* __restrict__ y, const float* H, int g,
+                                              int p, int64_t m0, int64_t m1, const Direction<D>* xi, const Window& v,
+                                              const int (&base)[SL], float* win, float* ring, bool more,
+                                              const f32x2* coef)
+{
+    constexpr int NT = interp_threads(D);
+    const int lane = threadIdx.x & 31;
+    for (int walk = 0; walk < v.walks; ++walk) {
+        const int nb = min(v.nb, v.nbt - walk * v.nb);
+        const int stride = (v.poly ? (nb + 1) * K + nb + W - 1 : nb + 2 * W) * 32;
         __syncthreads();
-        for (int64_t m = m0 + threadIdx.x; m < m1; m += blockDim.x) {
-            L.part[(size_t)s * L.M + m] = acc[m - m0];
-            L.part[(size_t)(L.S + s) * L.M + m] = acc[L.lane_T + (m - m0)];
+#pragma unroll
+        for (int h = 0; h < SL; ++h)
+            stage_cells<NT>(L, H + (size_t)min(p + 32 * h, L.P - 1) * L.G, p + 32 * h < L.P, base[h] + walk * v.nb, nb,
+                            v.poly, win + h * stride);
+        __syncthreads();
+        if (v.poly) {
+#pragma unroll 1
+            for (int h = 0; h < SL; ++h) form_polynomials<NT>(L, nb, win + h * stride);
+            __syncthreads();
+            interp_walk<D, SL, OUT, true>(L, y, g, m0, (int)(m1 - m0), xi, ring, win + lane, stride, v, base, walk, H, p, more || walk > 0, coef);
+        } else {
+            interp_walk<D, SL, OUT, false>(L, y, g, m0, (int)(m1 - m0), xi, ring, win + lane, stride, v, base, walk, H, p, more || walk > 0, coef);
+        }
+    }
+    __syncthreads();  // the window is done with
+}
+
+template <int D, int OUT>
+__global__ void __launch_bounds__(interp_threads(D), 1)
+    lane_interp_kernel(const __grid_constant__ qs_launch L, const float* __restrict__ y, const float* __restrict__ H,
+                       int win_bytes, int per_group)
+{
+    constexpr int SL = lane_slices(D);
+    extern __shared__ float4 smem4[];
+    unsigned char* sm = reinterpret_cast<unsigned char*>(smem4);
+    float* win = reinterpret_cast<float*>(smem4);
+    __shared__ int lohi[64 * SL];
+    __shared__ f32x2 coef[HW * T4];
+    share_coeffs(L.win, coef);  // read after the first barrier
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* ring = reinterpret_cast<float*>(sm + win_bytes) + warp * lane_ring_floats(D);
+    for (int i = lane; i < lane_ring_floats(D); i += 32) ring[i] = 0.0f;
+    const int G = L.G;
+    const int cap_poly = interp_cap_poly(win_bytes), cap_cells = interp_cap_cells(win_bytes);
+    const int64_t nblk = (L.M + 31) / 32;
+    int64_t b, b1;
+    cta_range(nblk * ((L.P + 32 * SL - 1) / (32 * SL)), nblk, per_group, b, b1);
+    while (b < b1) {
+        const int g = (int)(b / nblk);
+        const int64_t e = min(b1, (int64_t)(g + 1) * nblk);
+        const int64_t m0 = (b - (int64_t)g * nblk) * 32, m1 = min(L.M, (e - (int64_t)g * nblk) * 32);
+        b = e;
+        const int p = 32 * SL * g + lane;
+        Direction<D> xi[SL];
+#pragma unroll
+        for (int h = 0; h < SL; ++h) load_xi<D>(L, p + 32 * h, xi[h]);
+        sample_bins<D, interp_threads(D), SL>(L, y, g, m0, m1, xi, win, lohi);
+        int need[SL];
+#pragma unroll
+        for (int h = 0; h < SL; ++h) need[h] = sampled_need(lohi + 64 * h, G, lane);
+        if constexpr (SL == 2) {
+            const int most = max(need[0], need[1]);
+            const int cap_poly2 = interp_cap_poly(win_bytes / 2), cap_cells2 = interp_cap_cells(win_bytes / 2);
+            if (p - lane + 32 < L.P && pair_windows(most, cap_poly, cap_poly2, cap_cells2)) {
+                const Window v = place_window(most, cap_poly2, cap_cells2, false);
+                const int base[2] = {window_base(lohi, G, lane, v.nbt), window_base(lohi + 64, G, lane, v.nbt)};
+                interp_slices<D, 2, OUT>(L, y, H, g, p, m0, m1, xi, v, base, win, ring, false, coef);
+                continue;
+            }
+        }
+#pragma unroll 1
+        for (int h = 0; h < SL && p - lane + 32 * h < L.P; ++h) {
+            if (h) load_xi<D>(L, p + 32 * h, xi[0]);
+            // values written over their own projections allow one walk only
+            const Window v = place_window(h ? need[SL - 1] : need[0], cap_poly, cap_cells, OUT == 1 && D == 0);
+            const int base[1] = {window_base(lohi + 64 * h, G, lane, v.nbt)};
+            interp_slices<D, 1, OUT>(L, y, H, g, p + 32 * h, m0, m1, xi, v, base, win, ring, h > 0, coef);
         }
     }
 }
@@ -1007,42 +1191,59 @@ __global__ void __launch_bounds__(interp_threads(D), 1)
 // Dynamic shared memory of a CTA: all that the static 256 bytes leave.
 constexpr int LANE_SMEM = 226 * 1024;
 
+// How the work is cut: `group` units in each of `groups` slice groups, at least `least` per CTA; `visit` units
+// cost as much as placing, clearing and adding up a window.  A range of equal shares crosses into a second
+// group in some CTAs, which then set the time; whole CTAs per group leave some SMs out.
+struct Cut {
+    int ctas, per_group;
+};
+
+Cut cut_work(int64_t group, int64_t groups, int64_t least, double visit)
+{
+    const int64_t total = group * groups;
+    int64_t n = (total + least - 1) / least;
+    if (n > QS_LANE_CTAS) n = QS_LANE_CTAS;
+    const int64_t k = n / groups;
+    if (k < 1) return {(int)n, 0};
+    const double equal = (double)total / n + (n % groups ? 2.0 : 1.0) * visit;
+    const double whole = (double)((group + k - 1) / k) + visit;
+    return whole < equal ? Cut{(int)(k * groups), (int)k} : Cut{(int)n, 0};
+}
+
 template <int D>
 cudaError_t launch_spread_d(const qs_launch& L, const float* x, const float* w, int* Hi, cudaStream_t st)
 {
     const int win = (LANE_SMEM - lane_ring_bytes(D, spread_threads(D))) & ~1023;
     cudaError_t e = cudaFuncSetAttribute(lane_spread_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, LANE_SMEM);
     if (e != cudaSuccess) return e;
-    const int64_t total = (L.N + SUB - 1) / SUB * ((L.P + 31) / 32);
-    // at least 32 blocks of 8 points per CTA: fewer would not pay for its window
-    int64_t ctas = (total + 31) / 32;
-    if (ctas > QS_LANE_CTAS) ctas = QS_LANE_CTAS;
-    lane_spread_kernel<D><<<(unsigned)ctas, spread_threads(D), LANE_SMEM, st>>>(L, x, w, Hi, win);
+    // at least 32 blocks of 8 points per CTA: fewer would not pay for its window, which costs about 100
+    const Cut c = cut_work((L.N + SUB - 1) / SUB, (L.P + 32 * lane_slices(D) - 1) / (32 * lane_slices(D)), 32, 100.0);
+    lane_spread_kernel<D><<<(unsigned)c.ctas, spread_threads(D), LANE_SMEM, st>>>(L, x, w, Hi, win, c.per_group);
     return cudaGetLastError();
 }
 
 template <int D, int OUT>
 cudaError_t launch_interp_d(const qs_launch& L, const float* y, const float* H, cudaStream_t st)
 {
-    const int win = (LANE_SMEM - lane_ring_bytes(D, interp_threads(D)) - (OUT == 0 ? 8 * L.lane_T : 0)) & ~1023;
+    const int win = (LANE_SMEM - lane_ring_bytes(D, interp_threads(D))) & ~1023;
     cudaError_t e =
         cudaFuncSetAttribute(lane_interp_kernel<D, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, LANE_SMEM);
     if (e != cudaSuccess) return e;
-    const int64_t chunks = (L.m_end - L.m_base + L.lane_T - 1) / L.lane_T;
-    if (chunks <= 0) return cudaSuccess;
-    lane_interp_kernel<D, OUT><<<(unsigned)(chunks * L.S), interp_threads(D), LANE_SMEM, st>>>(L, y, H, win);
+    // at least 8 blocks of 32 targets per CTA, a window costs about 12
+    const Cut c = cut_work((L.M + 31) / 32, (L.P + 32 * lane_slices(D) - 1) / (32 * lane_slices(D)), 8, 12.0);
+    lane_interp_kernel<D, OUT><<<(unsigned)c.ctas, interp_threads(D), LANE_SMEM, st>>>(L, y, H, win, c.per_group);
     return cudaGetLastError();
 }
 
 }  // namespace
 
 // Coordinates per lane of the FP32 forms' kernels, 0 for the projections in U.
-static int lane_dims(const qs_launch& L, bool from_u)
+static int lane_dims(int d, bool from_u)
 {
     if (from_u) return 0;
     const int dims[] = {4, 8, 16, 32, 48, 64};
     for (int D : dims)
-        if (L.d <= D) return D;
+        if (d <= D) return D;
     return -1;
 }
 
@@ -1065,7 +1266,7 @@ cudaError_t qs_launch_lane_spread(const qs_launch& L, const float* x, const floa
                                   cudaStream_t st)
 {
     int* Hi = reinterpret_cast<int*>(grid);
-    switch (lane_dims(L, from_u)) {
+    switch (lane_dims(L.d, from_u)) {
         case 0: return launch_spread_d<0>(L, x, w, Hi, st);
         case 4: return launch_spread_d<4>(L, x, w, Hi, st);
         case 8: return launch_spread_d<8>(L, x, w, Hi, st);
@@ -1095,7 +1296,7 @@ cudaError_t qs_launch_lane_interp(const qs_launch& L, const float* y, bool from_
                                   cudaStream_t st)
 {
 #define QS_LANE_INTERP(DD) (deriv ? launch_interp_d<DD, 1>(L, y, H, st) : launch_interp_d<DD, 0>(L, y, H, st))
-    switch (lane_dims(L, from_u)) {
+    switch (lane_dims(L.d, from_u)) {
         case 0: return QS_LANE_INTERP(0);
         case 4: return QS_LANE_INTERP(4);
         case 8: return QS_LANE_INTERP(8);
@@ -1108,23 +1309,9 @@ cudaError_t qs_launch_lane_interp(const qs_launch& L, const float* y, bool from_
 #undef QS_LANE_INTERP
 }
 
-// Targets per CTA and slice groups of the interpolation: the fewest rounds of
-// (targets + the cost of staging a window, about 400 targets' worth) over the
-// CTAs, from M and P only.
-void qs_lane_shape(int64_t M, int P, int S_max, int* T, int* S)
+// Slice groups of the interpolation, a partial sum of each target for each.
+int qs_lane_groups(int P, int d, bool from_u)
 {
-    const int NG = (P + 31) / 32;
-    double best = 1e300;
-    for (int t = 256; t <= 4096; t = t < 1024 ? 2 * t : t + 1024) {
-        const int64_t chunks = (M + t - 1) / t;
-        for (int s = 1; s <= NG && s <= S_max; ++s) {
-            const int64_t rounds = (chunks * s + QS_LANE_CTAS - 1) / QS_LANE_CTAS;
-            const double cost = (double)rounds * ((NG + s - 1) / s) * (t + 400.0) + 2.0 * s;
-            if (cost < best) {
-                best = cost;
-                *T = t;
-                *S = s;
-            }
-        }
-    }
+    const int D = lane_dims(d, from_u), slices = 32 * (D < 0 ? 1 : lane_slices(D));
+    return (P + slices - 1) / slices;
 }

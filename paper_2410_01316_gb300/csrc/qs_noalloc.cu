@@ -217,18 +217,12 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     const size_t o_part = o_H + align256((size_t)P * G * 4);
     const size_t avail = o_part < QS_NOALLOC_SCRATCH_BYTES ? QS_NOALLOC_SCRATCH_BYTES - o_part : 0;
     while (S > 1 && (size_t)(2 * S) * (size_t)M * 4 > avail) --S;
-    // the slice-per-lane kernels by the rule of qs_sum, with as many slice groups as the scratch holds
+    // the slice-per-lane kernels by the rule of qs_sum, where the sums of their slice groups fit too
     const double span = G * qs_tau_rule(D.kernel, D.kparam, D.radius) * D.radius;
-    const bool lx = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, N, P, span),
-               ly = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, M, P, span);
-    int lane_T = 0;
-    if (ly) {
-        int lane_S = 1;
-        int64_t fit = (int64_t)(avail / 8) / M;
-        qs_lane_shape(M, P, (int)(fit < 1 ? 1 : (fit < S_max ? fit : S_max)), &lane_T, &lane_S);
-        S = lane_S;
-    }
-    const size_t need = o_part + (size_t)(2 * S) * (size_t)M * 4;
+    const int lane_S = qs_lane_groups(P, d, false);
+    const bool ly = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, M, P, span) && (size_t)lane_S * (size_t)M * 4 <= avail;
+    const bool lx = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, N, P, span);
+    const size_t need = o_part + (ly ? (size_t)lane_S : (size_t)(2 * S)) * (size_t)M * 4;
     if (need > QS_NOALLOC_SCRATCH_BYTES)
         return nfail(QS_ERR_UNSUPPORTED,
                      "qs_sum_noalloc: needs %zu bytes of scratch (P=%d, G=%d, M=%lld) but the static scratch "
@@ -254,7 +248,10 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     L.half_G = 0.5f * (float)G;
     L.U = nullptr;
     L.S = (int)S;
-    L.lane_T = lane_T;
+    if (ly) {
+        L.S = lane_S;
+        L.lane_part = true;
+    }
     L.spread_variant = qs_spread_default(G, W);
 
     unsigned char* base = nullptr;

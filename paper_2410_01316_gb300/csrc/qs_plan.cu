@@ -265,9 +265,12 @@ bool tensor_form(const qs_plan p) { return p->proj == QS_PROJ_BF16X3 || p->proj 
 // The same for the targets of a gradient, which the tensor-core forms back-project from BF16 parts.
 bool grad_lane(const qs_plan p, int64_t n) { return lane_use(p, n) && (!tensor_form(p) || p->d_qlo); }
 
-// The launch of the interpolation at M targets: lane_T and S of the slice-per-lane kernel, or S of the
-// point-per-lane one (make_launch's).
-void lane_launch(const qs_plan p, qs_launch* L) { qs_lane_shape(L->M, L->P, p->S_max, &L->lane_T, &L->S); }
+// The launch of the slice-per-lane interpolation and of the reduction after it.
+void lane_launch(const qs_plan p, qs_launch* L)
+{
+    L->S = qs_lane_groups(L->P, L->d, tensor_form(p));
+    L->lane_part = true;
+}
 
 // Operand preparation of the tensor-core forms (BF16 hi/lo split or TF32
 // rounding of the points into the plan's staging: the targets' own staging
@@ -564,7 +567,8 @@ qs_status qs_plan_create(qs_plan* out, const qs_plan_desc* desc)
     QS_ALLOC(p->d_H, (size_t)P * G);
     // slice-group partials: sized for targets up to max(max_n, max_m), since the
     // gradients evaluate at x as well as at y
-    QS_ALLOC(p->d_part, (size_t)2 * p->S_max * (maxnm > 0 ? maxnm : 1));
+    // (high and low parts of S_max groups, or sums of every 32 slices)
+    QS_ALLOC(p->d_part, (size_t)(2 * p->S_max > (P + 31) / 32 ? 2 * p->S_max : (P + 31) / 32) * (maxnm > 0 ? maxnm : 1));
     if (d <= QS_GRAD_MAX_D && proj == QS_PROJ_FP32_FUSED) {
         // per-component gradient partials of the fused form (the unfused forms
         // back-project with a GEMM): largest S(M) * M over M <= max(max_n, max_m), S as in make_launch
@@ -1001,7 +1005,6 @@ qs_status qs_grad(qs_plan p, const float* x, int64_t N, const float* w, const fl
             cudaError_t e1 = qs_launch_interp_deriv(L, p->W, p->d_H2, st);
             return e1 == cudaSuccess ? qs_launch_backproj(p->d_U, p->ldU, L.M, L.P, p->d_dirs, d, scale, fac, out, st) : e1;
         }
-        qs_lane_shape(L.M, L.P, (L.P + 31) / 32, &L.lane_T, &L.S);  // no partial sums: any number of groups
         L.Qlo = p->d_qlo;
         e = qs_launch_lane_interp(L, pts, from_u, p->d_H2, true, st);
         if (e != cudaSuccess) return e;
