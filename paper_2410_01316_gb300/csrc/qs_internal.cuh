@@ -39,7 +39,6 @@ constexpr int QS_INLINE_WEIGHTS = 4096;        // most sources whose weights the
 // Slice-per-lane grid kernels (qs_lane.cu): the default window width only.
 constexpr int QS_LANE_W = 8;
 constexpr int QS_LANE_CTAS = 152;              // CTAs that the work is cut into: one per SM
-constexpr int64_t QS_LANE_MIN_PAIRS = 1 << 20;
 constexpr int QS_PREP_BLOCKS = 152;            // most blocks of the weight bound
 // wscale: scale, inverse, max |w| scale, non-finite; 2 partials per block; the ticket
 constexpr int QS_WSCALE_FLOATS = 4 + 2 * QS_PREP_BLOCKS + 4;
@@ -364,5 +363,9 @@ inline bool qs_lane_use(qs_proj proj, int W, int d, int64_t n, int P, double spa
     if (W != QS_LANE_W || (proj == QS_PROJ_FP32 && d > QS_FUSED_MAX_D)) return false;
     const double sigmas = 4.2 / sqrt((double)d);
     if (span * (sigmas < 1.0 ? sigmas : 1.0) > 1600.0) return false;
-    return n >= 512 && n < ((int64_t)1 << 31) && n * (int64_t)P >= QS_LANE_MIN_PAIRS;
+    // placing, clearing and adding up the windows takes 10 to 30 us, the more the more coordinates a lane
+    // holds: even with the point-per-lane kernels at 1e6 pairs with projections from U or d <= 4 (d = 64:
+    // 78 us either way; at 2e6 84 against 88), 4e6 at d = 16, 6e6 at d = 30
+    const int64_t least = proj == QS_PROJ_BF16X3 || proj == QS_PROJ_TF32 || d <= 4 ? 2 << 20 : (d <= 16 ? 3 << 20 : 6 << 20);
+    return n >= 512 && n < ((int64_t)1 << 31) && n * (int64_t)P >= least;
 }

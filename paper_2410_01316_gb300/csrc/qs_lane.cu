@@ -147,13 +147,29 @@ struct Direction {
     f32x2 c[D > 0 ? D / 2 : 1];
 };
 
-template <int D>
-__device__ __forceinline__ void load_xi(const qs_launch& L, int p, Direction<D>& xi)
+// The directions of the group's slices, lane l's at p0 + 32 h + l, by way of shared memory: read by every
+// lane from global memory they would cost each warp 32 lines per coordinate (12 us of a CTA of 12 warps at
+// d = 30).  scratch: 32 SL (D + 1) floats.  Begins and ends with a barrier.
+template <int D, int SL>
+__device__ __forceinline__ void share_xi(const qs_launch& L, int p0, Direction<D>* xi, float* scratch)
 {
-    const float* src = L.xi_s + (size_t)p * L.d;
-    auto at = [&](int j) { return (p < L.P && j < L.d) ? __ldg(&src[j]) : 0.0f; };
+    if constexpr (D > 0) {
+        const int lane = threadIdx.x & 31, d = L.d, rows = min(32 * SL, L.P - p0);
+        const float* src = L.xi_s + (size_t)p0 * d;
+        __syncthreads();
+        for (int e = threadIdx.x; e < 32 * SL * d; e += blockDim.x) {
+            const int r = e / d;
+            scratch[r * (D + 1) + (e - r * d)] = r < rows ? __ldg(&src[e]) : 0.0f;
+        }
+        __syncthreads();
 #pragma unroll
-    for (int j = 0; j < D; j += 2) xi.c[j / 2] = pack2(at(j), at(j + 1));
+        for (int h = 0; h < SL; ++h) {
+            const float* row = scratch + (32 * h + lane) * (D + 1);
+#pragma unroll
+            for (int j = 0; j < D; j += 2) xi[h].c[j / 2] = pack2(j < d ? row[j] : 0.0f, j + 1 < d ? row[j + 1] : 0.0f);
+        }
+        __syncthreads();
+    }
 }
 
 // Grid coordinates of the staged point at r on the lane's slices: FP32 products summed in four strands
@@ -347,13 +363,6 @@ __device__ __forceinline__ Window place_window(int need, int cap_poly, int cap_c
     }
     v.nb = (v.nbt + v.walks - 1) / v.walks;
     return v;
-}
-
-// Two slices per lane where two windows of polynomials fit, or, for spans too wide for one of polynomials,
-// two of cells.
-__device__ __forceinline__ bool pair_windows(int need, int cap_poly, int cap_poly2, int cap_cells2)
-{
-    return need <= cap_poly2 || (need > cap_poly && need <= cap_cells2);
 }
 
 // ---------------------------------------------------------------------------
@@ -777,8 +786,7 @@ __global__ void __launch_bounds__(spread_threads(D), 1)
         b = e;
         const int p = 32 * SL * g + lane;
         Direction<D> xi[SL];
-#pragma unroll
-        for (int h = 0; h < SL; ++h) load_xi<D>(L, p + 32 * h, xi[h]);
+        share_xi<D, SL>(L, p - lane, xi, reinterpret_cast<float*>(c.win));
         sample_bins<D, spread_threads(D), SL>(L, x, g, 0, L.N, xi, reinterpret_cast<float*>(c.win), lohi);
         int need[SL];
 #pragma unroll
@@ -786,7 +794,7 @@ __global__ void __launch_bounds__(spread_threads(D), 1)
         if constexpr (SL == 2) {
             const int most = max(need[0], need[1]);
             const int cap_poly2 = win_bytes / 2 / (K * 128) - 1, cap_cells2 = win_bytes / 2 / 128 - (2 * W - 1);
-            if (p - lane + 32 < L.P && pair_windows(most, cap_poly, cap_poly2, cap_cells2)) {
+            if (p - lane + 32 < L.P && most <= cap_cells2) {
                 const Window v = place_window(most, cap_poly2, cap_cells2, false);
                 const int base[2] = {window_base(lohi, G, lane, v.nbt), window_base(lohi + 64, G, lane, v.nbt)};
                 spread_slices<D, 2>(L, c, g, p, n0, n1, xi, v, base);
@@ -795,7 +803,7 @@ __global__ void __launch_bounds__(spread_threads(D), 1)
         }
 #pragma unroll 1
         for (int h = 0; h < SL && p - lane + 32 * h < L.P; ++h) {
-            if (h) load_xi<D>(L, p + 32 * h, xi[0]);
+            if (h) share_xi<D, 1>(L, p - lane + 32 * h, xi, reinterpret_cast<float*>(c.win));
             const Window v = place_window(h ? need[SL - 1] : need[0], cap_poly, cap_cells, false);
             const int base[1] = {window_base(lohi + 64 * h, G, lane, v.nbt)};
             spread_slices<D, 1>(L, c, g, p + 32 * h, n0, n1, xi, v, base);
@@ -1161,8 +1169,7 @@ __global__ void __launch_bounds__(interp_threads(D), 1)
         b = e;
         const int p = 32 * SL * g + lane;
         Direction<D> xi[SL];
-#pragma unroll
-        for (int h = 0; h < SL; ++h) load_xi<D>(L, p + 32 * h, xi[h]);
+        share_xi<D, SL>(L, p - lane, xi, win);
         sample_bins<D, interp_threads(D), SL>(L, y, g, m0, m1, xi, win, lohi);
         int need[SL];
 #pragma unroll
@@ -1170,7 +1177,7 @@ __global__ void __launch_bounds__(interp_threads(D), 1)
         if constexpr (SL == 2) {
             const int most = max(need[0], need[1]);
             const int cap_poly2 = interp_cap_poly(win_bytes / 2), cap_cells2 = interp_cap_cells(win_bytes / 2);
-            if (p - lane + 32 < L.P && pair_windows(most, cap_poly, cap_poly2, cap_cells2)) {
+            if (p - lane + 32 < L.P && most <= cap_cells2) {
                 const Window v = place_window(most, cap_poly2, cap_cells2, false);
                 const int base[2] = {window_base(lohi, G, lane, v.nbt), window_base(lohi + 64, G, lane, v.nbt)};
                 interp_slices<D, 2, OUT>(L, y, H, g, p, m0, m1, xi, v, base, win, ring, false, coef);
@@ -1179,7 +1186,7 @@ __global__ void __launch_bounds__(interp_threads(D), 1)
         }
 #pragma unroll 1
         for (int h = 0; h < SL && p - lane + 32 * h < L.P; ++h) {
-            if (h) load_xi<D>(L, p + 32 * h, xi[0]);
+            if (h) share_xi<D, 1>(L, p - lane + 32 * h, xi, win);
             // values written over their own projections allow one walk only
             const Window v = place_window(h ? need[SL - 1] : need[0], cap_poly, cap_cells, OUT == 1 && D == 0);
             const int base[1] = {window_base(lohi + 64 * h, G, lane, v.nbt)};

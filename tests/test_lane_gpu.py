@@ -1,4 +1,4 @@
-"""The slice-per-lane grid stages (sums and gradients of at least 2^20 (point, slice) pairs).
+"""The slice-per-lane grid stages (sums and gradients of at least 2 to 6 million (point, slice) pairs).
 
 Every branch of their dispatch against the FP64 oracle: coordinates per lane (d = 1 .. 64) or projections
 from the tensor cores, polynomials or plain cells per window, several windows per slice, points outside the
@@ -74,18 +74,18 @@ def _check(prob, proj, grads=True, plan_kw=None, shift=0):
         assert np.max(np.abs(g["w"][jn] - rg["w"])) / (sv * maxF) < tol
 
 
-@pytest.mark.parametrize("d,P,N,M,proj", [(1, 33, 32003, 31777, "fp32_fused"), (3, 100, 10487, 10501, "auto"),
-                                          (4, 64, 16384, 16391, "fp32"), (5, 96, 11003, 12001, "fp32"),
-                                          (16, 130, 9001, 8111, "fp32"), (30, 100, 10500, 10499, "fp32"),
-                                          (40, 128, 8200, 8195, "fp32"), (64, 65, 17001, 16501, "fp32"),
-                                          (64, 200, 5301, 5303, "bf16x3"), (100, 97, 11003, 10903, "bf16x3"),
-                                          (300, 64, 16601, 16433, "bf16x3")])
+@pytest.mark.parametrize("d,P,N,M,proj", [(1, 33, 64003, 63777, "fp32_fused"), (3, 100, 20983, 21001, "auto"),
+                                          (4, 64, 32768, 32775, "fp32"), (5, 96, 33003, 34001, "fp32"),
+                                          (16, 130, 26001, 24311, "fp32"), (30, 100, 63000, 62999, "fp32"),
+                                          (20, 192, 33001, 33003, "fp32"), (40, 128, 50400, 50387, "fp32"), (64, 65, 98001, 97001, "fp32"),
+                                          (64, 200, 10501, 10503, "bf16x3"), (100, 97, 22003, 21703, "bf16x3"),
+                                          (300, 64, 33001, 32801, "bf16x3")])
 def test_dimensions_and_ragged_sizes(d, P, N, M, proj):
     prob = W.tiny(d=d, N=N, M=M, P=P, kernel="gauss", kparam=1.1 * np.sqrt(2 * d), n_ft=128, seed=d + P)
     _check(prob, proj)
 
 
-@pytest.mark.parametrize("n_ft,P,N", [(256, 40, 27000), (1024, 34, 31000), (2048, 32, 33000)])
+@pytest.mark.parametrize("n_ft,P,N", [(256, 70, 90000), (1024, 66, 96000), (2048, 64, 99000)])
 @pytest.mark.parametrize("proj", ["fp32_fused", "bf16x3"])
 def test_wide_windows_and_several_per_slice(n_ft, P, N, proj):
     # negative distance in d = 40 with one set nearly filling the radius along two axes, so that its
@@ -105,7 +105,7 @@ def test_wide_windows_and_several_per_slice(n_ft, P, N, proj):
 @pytest.mark.parametrize("proj", ["fp32", "bf16x3"])
 def test_points_outside_the_sampled_window(proj):
     # most points in a narrow cluster, a few far out that a sample of 256 mostly misses
-    prob = W.tiny(d=16, N=16500, M=16600, P=70, kernel="gauss", kparam=3.0, n_ft=512, seed=9)
+    prob = W.tiny(d=16, N=46000, M=46200, P=70, kernel="gauss", kparam=3.0, n_ft=512, seed=9)
     for a in (prob.x, prob.y):
         a *= 0.1
         a[np.random.default_rng(3).choice(len(a), 25, replace=False)] *= 60.0
@@ -115,7 +115,7 @@ def test_points_outside_the_sampled_window(proj):
 
 @pytest.mark.parametrize("weights", ["none", "one", "tiny", "zeros", "mixed"])
 def test_weights(weights):
-    prob = W.tiny(d=5, N=12000, M=11000, P=100, kernel="laplace", kparam=0.6, n_ft=256, seed=4)
+    prob = W.tiny(d=5, N=34000, M=32000, P=100, kernel="laplace", kparam=0.6, n_ft=256, seed=4)
     if weights == "none":
         prob.w = None
     elif weights == "one":  # one weight outweighs all others: the windows' conversions leave the fast range
@@ -138,7 +138,7 @@ def test_weights(weights):
 
 @pytest.mark.parametrize("d", [3, 4, 6, 16, 30])
 def test_unaligned_inputs(d):
-    prob = W.tiny(d=d, N=11001, M=11003, P=100, kernel="gauss", kparam=2.0 * np.sqrt(d), n_ft=128, seed=d)
+    prob = W.tiny(d=d, N=32001, M=32003, P=200 if d > 16 else 100, kernel="gauss", kparam=2.0 * np.sqrt(d), n_ft=128, seed=d)
     _check(prob, "fp32", shift=1)
 
 
@@ -146,7 +146,7 @@ def test_unaligned_inputs(d):
 def test_data_errors_are_flagged(proj):
     import torch
 
-    prob = W.tiny(d=16, N=12000, M=11000, P=100, kernel="gauss", kparam=6.0, n_ft=256, seed=6)
+    prob = W.tiny(d=16, N=34000, M=32000, P=100, kernel="gauss", kparam=6.0, n_ft=256, seed=6)
     x, w, y = _cuda(prob.x), _cuda(prob.w), _cuda(prob.y)
     with QSPlan(16, "gauss", prob.P, prob.n_ft, prob.R, prob.kparam, dirs=prob.xi, proj=proj, max_n=prob.N,
                 max_m=prob.M) as plan:
