@@ -113,7 +113,7 @@ def test_points_outside_the_sampled_window(proj):
     _check(prob, proj)
 
 
-@pytest.mark.parametrize("weights", ["none", "one", "tiny", "zeros", "mixed"])
+@pytest.mark.parametrize("weights", ["none", "one", "tiny", "tiniest", "zeros", "mixed"])
 def test_weights(weights):
     prob = W.tiny(d=5, N=34000, M=32000, P=100, kernel="laplace", kparam=0.6, n_ft=256, seed=4)
     if weights == "none":
@@ -122,6 +122,8 @@ def test_weights(weights):
         prob.w[77] = 1e6
     elif weights == "tiny":
         prob.w *= np.float32(1e-30)
+    elif weights == "tiniest":  # the grid's scale is close to the largest number: no finer windows
+        prob.w *= np.float32(3e-34)
     elif weights == "mixed":
         prob.w *= np.exp(np.random.default_rng(3).uniform(-12, 0, prob.N)).astype(np.float32)
     else:
