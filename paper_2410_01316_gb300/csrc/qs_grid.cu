@@ -1265,8 +1265,9 @@ __global__ void __launch_bounds__(256) reduce_grad_kernel(const float* __restric
     if (strip == 0 && i < M * d) out[i] = (hi + lo) * scale * (fac ? __ldg(&fac[i / d]) : 1.0f);
 }
 
-// Strips pay while a block per 256 elements leaves SMs idle and a strip still has groups to load.
-bool reduce_in_strips(int S, int64_t n) { return S >= 16 && n <= (int64_t)QS_LANE_CTAS * 256; }
+// Strips pay while one strip's blocks of 256 elements (at most 8 per SM) do not hide its rounds of loads and a
+// strip still has groups to load (60000 targets: the stage 16.4 us in one strip, 10.2 in strips).
+bool reduce_in_strips(int S, int64_t n) { return S >= 16 && n <= (int64_t)QS_LANE_CTAS * 2048; }
 
 // Opt-in to `smem` bytes of dynamic shared memory, where that and up to 10 KB of static shared memory
 // pass the 48 KB that need none (the call costs about a microsecond of the host's time).
