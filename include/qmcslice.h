@@ -83,7 +83,8 @@ typedef enum {
 /* Precision / form of the projection step a = tau X Xi^T. */
 typedef enum {
     QS_PROJ_AUTO = 0,       /* fused for d <= 4, FP32 for d < 64, BF16x3 from d = 64 */
-    QS_PROJ_FP32 = 1,       /* FP32 SIMT GEMM into a P x N workspace */
+    QS_PROJ_FP32 = 1,       /* FP32 SIMT GEMM into a P x N workspace; inside the grid kernels
+                               for large problems with W = 8 and d <= 64 */
     QS_PROJ_FP32_FUSED = 2, /* FP32 dot products inside spread / interpolation (d <= 64) */
     QS_PROJ_BF16X3 = 3,     /* tensor-core GEMM, x = hi + lo split in BF16, three products */
     QS_PROJ_TF32 = 4        /* tensor-core GEMM in TF32 */
@@ -169,7 +170,9 @@ qs_status qs_sum(qs_plan plan, const float* x, int64_t N, const float* w,
  * swap roles with y and v).  The unfused projection forms (QS_PROJ_FP32,
  * QS_PROJ_BF16X3, QS_PROJ_TF32) write the derivative values of every
  * (point, slice) pair over the plan's projection buffer and back-project them
- * by a GEMM (points x P)(P x d) with compensated slice-chunk sums; the fused
+ * by a GEMM (points x P)(P x d): FP32 with compensated slice-chunk sums, or, for
+ * large problems in the tensor-core forms, six products of three-way BF16
+ * splits with FP32 sums over chunks of 64 slices; the fused
  * form, which has no projection buffer, sums the back-projection inside the
  * interpolation per component and so needs d <= 32.  x: N x d,
  * w: N (NULL = ones), y: M x d, v: M (NULL = ones), gx: N x d, gw: N,
@@ -196,7 +199,8 @@ qs_status qs_project(qs_plan plan, const float* x, int64_t N, float* u_out, int6
  * synchronises `stream`.  The copies in run on a plan-owned copy stream in
  * row chunks (at most 8 for x and 2 for y, after the work already queued on
  * `stream`), and each chunk is projected on `stream` as soon as it has
- * landed (each target chunk also interpolated), so the transfers overlap the
+ * landed (each target chunk also interpolated, except where large problems take one
+ * interpolation for all targets), so the transfers overlap the
  * projections, the spread and the interpolation; the result is the one
  * qs_sum computes, bit for bit.  With
  * stage timing on (qs_set_timing) or N == 0 the copies run first, on
@@ -371,6 +375,8 @@ qs_status qs_batch_autotune(qs_batch batch, const qs_problem* probs, int* chosen
  * copies; 3: a 32-cell window with one column per thread plus one grid).
  * Within a family the variants produce bitwise identical results and differ
  * only in speed, which depends on how the projections cluster.
+ * They apply where the spread has one point per lane; large problems with
+ * W = 8 are spread with one slice per lane, which has no variants.
  * qs_plan_autotune runs the spread of the given sources once per variant of
  * the family (timed with CUDA events on `stream`, best of 3 after a warm-up),
  * keeps the fastest in the plan and writes its index to *chosen (may be
