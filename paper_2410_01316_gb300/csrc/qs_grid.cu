@@ -145,34 +145,45 @@ __global__ void __launch_bounds__(1024) weight_scale_kernel(const float* __restr
 
 // The fixed-point scale and its inverse: from weight_scale_kernel, or, for the
 // few sources of a small problem (QS_INLINE_WEIGHTS), summed by every CTA of
-// the spread itself (the same sum in each): a microsecond of loads and a block
-// reduction there against a launch of 3.5 us ahead of it.  sc: two floats of
+// the spread itself: a microsecond of loads and a block reduction there against
+// a launch of 3.5 us ahead of it.  The sum is taken in that kernel's order
+// (thread t stands for its threads t, t + blockDim.x, ...; blockDim.x divides
+// 1024), bit for bit: another last bit of the scale rounds every contribution
+// to the grid anew, 1e-6 of a result whose weights cancel.  sc: two floats of
 // shared memory; ends with a barrier in the second case.
 __device__ __forceinline__ float2 slice_scale(const qs_launch& L, const float* __restrict__ w, float* sc)
 {
     if (L.N > QS_INLINE_WEIGHTS) return make_float2(__ldg(&L.wscale[0]), __ldg(&L.wscale[1]));
-    __shared__ float red[32];
-    float acc = 0.0f;
-    if (w)
-        for (int n = threadIdx.x; n < (int)L.N; n += blockDim.x) acc += fabsf(__ldg(&w[n]));
+    constexpr int NT = 1024;  // threads of weight_scale_kernel
+    __shared__ float red[NT / 32];
+    const int lane = threadIdx.x & 31;
+    if (w) {
+        for (int t = threadIdx.x; t < NT; t += blockDim.x) {
+            float acc = 0.0f;
+            for (int n = t; n < (int)L.N; n += NT) acc += fabsf(__ldg(&w[n]));
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float B = 0.0f;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) B += red[i];
-        if (!w) B = (float)L.N;
-        float scale = 0.0f, inv = 0.0f;
-        if (!isfinite(B)) {
-            atomicOr(L.flag, QS_FLAG_NONFINITE);
-        } else if (B > 0.0f) {
-            scale = 1073741824.0f / B;
-            inv = B / 1073741824.0f;
-            if (!isfinite(scale)) scale = inv = 0.0f;  // B below 2^-98: all weights negligible
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) red[t >> 5] = acc;
         }
-        sc[0] = scale;
-        sc[1] = inv;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        float B = w ? red[lane] : 0.0f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) B += __shfl_xor_sync(0xffffffffu, B, o);
+        if (lane == 0) {
+            if (!w) B = (float)L.N;
+            float scale = 0.0f, inv = 0.0f;
+            if (!isfinite(B)) {
+                atomicOr(L.flag, QS_FLAG_NONFINITE);
+            } else if (B > 0.0f) {
+                scale = 1073741824.0f / B;
+                inv = B / 1073741824.0f;
+                if (!isfinite(scale)) scale = inv = 0.0f;  // B below 2^-98: all weights negligible
+            }
+            sc[0] = scale;
+            sc[1] = inv;
+        }
     }
     __syncthreads();
     return make_float2(sc[0], sc[1]);
