@@ -385,6 +385,13 @@ qs_status qs_batch_autotune(qs_batch batch, const qs_problem* probs, int* chosen
  */
 qs_status qs_plan_autotune(qs_plan plan, const float* x, int64_t N, const float* w, int* chosen, void* stream);
 /*
+ * Which kind of grid kernels a sum of this plan uses for n points (sources:
+ * the spread; targets: the interpolation): *lanes = 1 for one slice per lane,
+ * 0 for one point per lane.  A function of the plan and n alone.  The kinds
+ * agree within the sums' accuracy, not bit for bit.
+ */
+qs_status qs_plan_lanes(qs_plan plan, int64_t n, int* lanes);
+/*
  * Projection GEMM form by timing (tensor-core plans): runs the projection of
  * the N points in x (device, N x d) with one CTA per SM and, where two-CTA
  * clusters can be resident, on SM pairs (best of 3 after a warm-up, CUDA

@@ -192,6 +192,12 @@ class QSPlan:
         _lib.check(self._lib.qs_plan_variants(self._handle, None, ctypes.byref(cur)), "qs_plan_variants")
         return self.SPREAD_VARIANTS[cur.value]
 
+    def lanes(self, n: int) -> bool:
+        """Whether sums of this plan run their grid stages of n points with one slice per lane."""
+        v = ctypes.c_int(-1)
+        _lib.check(self._lib.qs_plan_lanes(self._handle, n, ctypes.byref(v)), "qs_plan_lanes")
+        return v.value == 1
+
     # -- stage timing -----------------------------------------------------
     STAGES = ("prep_x", "project_x", "spread_filter", "prep_y", "project_y", "interp", "reduce")
 

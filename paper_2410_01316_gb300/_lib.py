@@ -36,7 +36,7 @@ EXPORTS = ("qs_plan_create", "qs_plan_destroy", "qs_plan_info", "qs_plan_directi
            "qs_batch_check", "qs_batch_set_tiling", "qs_plan_variants", "qs_distance_design",
            "qs_distance_energy", "qs_sum_sorted", "qs_grad_sorted", "qs_plan_set_gemm", "qs_plan_gemm",
            "qs_sobol_points", "qs_batch_autotune", "qs_plan_autotune_gemm", "qs_tune_cache_save",
-           "qs_tune_cache_load", "qs_tune_cache_clear", "qs_tune_cache_size", "qs_batch_set_mode")
+           "qs_tune_cache_load", "qs_tune_cache_clear", "qs_tune_cache_size", "qs_batch_set_mode", "qs_plan_lanes")
 
 
 class PlanDesc(ctypes.Structure):
@@ -100,6 +100,7 @@ def load() -> ctypes.CDLL:
         lib.qs_plan_set_variant.argtypes = [c_vp, c_int]
         lib.qs_plan_set_gemm.argtypes = [c_vp, c_int]
         lib.qs_plan_gemm.argtypes = [c_vp, ctypes.POINTER(c_int), ctypes.POINTER(c_int)]
+        lib.qs_plan_lanes.argtypes = [c_vp, c_i64, ctypes.POINTER(c_int)]
         lib.qs_plan_variants.argtypes = [c_vp, ctypes.POINTER(ctypes.c_uint), ctypes.POINTER(c_int)]
         lib.qs_distance_design.argtypes = [c_vp, c_int, c_int, c_int, c_dbl, ctypes.POINTER(c_dbl), c_vp]
         lib.qs_distance_energy.argtypes = [c_vp, c_int, c_int, ctypes.POINTER(c_dbl), c_vp, c_vp]
@@ -118,7 +119,7 @@ def load() -> ctypes.CDLL:
                      "qs_batch_set_tiling", "qs_plan_variants", "qs_distance_design", "qs_distance_energy",
                      "qs_sum_sorted", "qs_grad_sorted", "qs_plan_set_gemm", "qs_plan_gemm", "qs_sobol_points",
                      "qs_batch_autotune", "qs_plan_autotune_gemm", "qs_tune_cache_save", "qs_tune_cache_load",
-                     "qs_tune_cache_clear", "qs_tune_cache_size", "qs_batch_set_mode"):
+                     "qs_tune_cache_clear", "qs_tune_cache_size", "qs_batch_set_mode", "qs_plan_lanes"):
             getattr(lib, name).restype = c_int
         _lib = lib
         return lib

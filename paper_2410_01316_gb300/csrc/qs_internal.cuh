@@ -40,6 +40,9 @@ constexpr int QS_INLINE_WEIGHTS = 4096;        // most sources whose weights the
 constexpr int QS_LANE_W = 8;
 constexpr int QS_LANE_CTAS = 152;              // CTAs that the work is cut into: one per SM
 constexpr int QS_PREP_BLOCKS = 152;            // most blocks of the weight bound
+// Up to QS_LANE_FEW slices the slice-per-lane kernels take QS_LANE_FEW_POINTS points: see qs_lane_use
+constexpr int QS_LANE_FEW = 256;
+constexpr int QS_LANE_FEW_POINTS = 48 << 10;
 // wscale: scale, inverse, max |w| scale, non-finite; 2 partials per block; the ticket
 constexpr int QS_WSCALE_FLOATS = 4 + 2 * QS_PREP_BLOCKS + 4;
 
@@ -363,6 +366,13 @@ inline bool qs_lane_use(qs_proj proj, int W, int d, int64_t n, int P, double spa
     if (W != QS_LANE_W || (proj == QS_PROJ_FP32 && d > QS_FUSED_MAX_D)) return false;
     const double sigmas = 4.2 / sqrt((double)d);
     if (span * (sigmas < 1.0 ? sigmas : 1.0) > 1600.0) return false;
+    // Few slices and not many points: the problems of which batches are made.  Their pipelines run side by
+    // side, and kernels that take whole SMs then gain nothing (48 uneven problems of P = 128 / 256 in one call:
+    // up to 12000 points 0.99 / 1.00x, up to 30000 0.98 / 1.02x, up to 40000 1.04 / 1.07x; a sum of 20000 x 20000
+    // alone 0.97 to 1.00x at P = 128, 1.0 to 1.19x at P = 256).  So they keep the point-per-lane kernels, and with
+    // them their results: with few slices to average over, the two kinds differ by the rounding of the
+    // point-per-lane spread to sum |w| 2^-30, up to 3e-5 of a result whose weights cancel.
+    if (P <= QS_LANE_FEW && n < QS_LANE_FEW_POINTS) return false;
     // placing, clearing and adding up the windows takes 10 to 30 us, the more the more coordinates a lane
     // holds: even with the point-per-lane kernels at 1e6 pairs with projections from U or d <= 4 (d = 64:
     // 78 us either way; at 2e6 84 against 88), 4e6 at d = 16, 6e6 at d = 30

@@ -1083,6 +1083,13 @@ qs_status qs_plan_gemm(qs_plan p, int* pair, int* ctas)
     return QS_OK;
 }
 
+qs_status qs_plan_lanes(qs_plan p, int64_t n, int* lanes)
+{
+    if (!p || !lanes || n < 0) return fail(QS_ERR_ARG, "qs_plan_lanes: bad argument");
+    *lanes = lane_use(p, n) ? 1 : 0;
+    return QS_OK;
+}
+
 qs_status qs_plan_variants(qs_plan p, unsigned int* available, int* current)
 {
     if (!p) return fail(QS_ERR_ARG, "qs_plan_variants: NULL plan");
