@@ -104,17 +104,12 @@ __device__ __forceinline__ void fft_pass(float2* z, int n, int len, const float2
 #pragma unroll
         for (int q = 0; q < R; ++q) v[q] = z[fft_sw(base + q * sub)];
         if (sub > 1) {
-            // w^q from the table for q = 1, 2, 4 (indices below G/2), the others by one product
-            w[1] = __ldg(&tw[j * ts]);
-            if (R > 2) {
-                w[2] = __ldg(&tw[2 * j * ts]);
-                w[3] = cmul(w[1], w[2]);
-            }
-            if constexpr (R == 8) {
-                w[4] = __ldg(&tw[4 * j * ts]);
-                w[5] = cmul(w[1], w[4]);
-                w[6] = cmul(w[2], w[4]);
-                w[7] = cmul(w[3], w[4]);
+            // w^q, all from the table (a product of two entries would round twice more); entry t + G/2 is minus entry t
+#pragma unroll
+            for (int q = 1; q < R; ++q) {
+                const int t = q * j * ts, h = G >> 1;
+                w[q] = __ldg(&tw[t & (h - 1)]);
+                if (2 * q > R && t >= h) w[q] = make_float2(-w[q].x, -w[q].y);
             }
         }
         if (INV && sub > 1) {
