@@ -1541,8 +1541,8 @@ cudaError_t qs_launch_reduce(const qs_launch& L, float* s, cudaStream_t st)
 {
     const bool strips = reduce_in_strips(L.S, L.M);
     const unsigned grid = (unsigned)(strips ? (L.M + RS_ELEMS - 1) / RS_ELEMS : (L.M + 255) / 256);
-    auto kern = strips ? (L.lane_part ? reduce_kernel<RS_STRIPS, false> : reduce_kernel<RS_STRIPS, true>)
-                       : (L.lane_part ? reduce_kernel<1, false> : reduce_kernel<1, true>);
+    auto kern = strips ? (L.no_low ? reduce_kernel<RS_STRIPS, false> : reduce_kernel<RS_STRIPS, true>)
+                       : (L.no_low ? reduce_kernel<1, false> : reduce_kernel<1, true>);
     kern<<<grid, 256, 0, st>>>(L.part, L.S, L.M, L.P, s);
     return cudaGetLastError();
 }

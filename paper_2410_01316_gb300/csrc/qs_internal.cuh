@@ -111,7 +111,7 @@ struct qs_launch {
     float* part;          // 2 x S x M partial slice sums (hi, lo)
     int S;                // number of slice groups of the interpolation
     void* Qlo;            // low BF16 parts of the derivative values (tensor-core forms), [p / 32][m][32]
-    bool lane_part;       // part holds the slice-per-lane interpolation's sums: S x M, no low parts
+    bool no_low;          // part holds S x M sums, no low parts (slice-per-lane interpolation without room for them)
     unsigned int* flag;   // device error flag
     float* wscale;        // [0] = 2^30 / sum|w| (fixed-point scale of the grids), [1] = its inverse; QS_WSCALE_FLOATS
     int spread_variant;   // QS_SPREAD_* (all variants give bitwise identical grids)

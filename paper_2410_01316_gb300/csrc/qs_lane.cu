@@ -866,17 +866,34 @@ __global__ void __launch_bounds__(256) lane_filter_kernel(const __grid_constant_
 // (A grid of target chunks x group ranges left 39 % of the SM time idle at
 // 2e4 targets and 32 groups, and staged a window per group and chunk.)  The 32
 // values of a target are added across the lanes as the targets go by -- pairs
-// of targets over lane bit 0, pairs of pairs over bit 1, and so on, one shuffle
-// per target in all -- after which lane l holds the group's sum of target l of
-// the block, written to part[g][m]; the groups' sums are accumulated by TwoSum
-// in increasing order by the reduction.
+// of targets over lane bit 0, pairs of pairs over bit 1, and so on, one to two
+// shuffles per target in all -- after which lane l holds the group's sum of target
+// l of the block.  Every addition is a TwoSum, its error goes along (2.5 to 5 % of
+// a sum's time against plain additions; two sums side by side in packed
+// arithmetic: 1 % less at d = 64 and 784, 2 % more at d = 30, not kept): hi to
+// part[g][m] and lo to part[S + g][m] (without room for low parts, P > 2048 slices,
+// hi + lo to part[g][m]); the reduction accumulates the groups the same way.
 // ---------------------------------------------------------------------------
-template <int B>
-__device__ __forceinline__ float fold(float a, float b, int lane)
+struct Sum {
+    float hi, lo;  // the rounding errors of all additions so far in lo
+};
+
+__device__ __forceinline__ void add(Sum& a, Sum b)
+{
+    qs_two_sum(a.hi, a.lo, b.hi);
+    a.lo += b.lo;
+}
+
+// LOW: the values have low parts.
+template <int B, bool LOW = true>
+__device__ __forceinline__ Sum fold(Sum a, Sum b, int lane)
 {
     const bool up = (lane >> B) & 1;
-    const float keep = up ? b : a, send = up ? a : b;
-    return keep + __shfl_xor_sync(0xffffffffu, send, 1 << B);
+    Sum keep = {up ? b.hi : a.hi, LOW ? (up ? b.lo : a.lo) : 0.0f}, other = {up ? a.hi : b.hi, 0.0f};
+    other.hi = __shfl_xor_sync(0xffffffffu, other.hi, 1 << B);
+    if (LOW) other.lo = __shfl_xor_sync(0xffffffffu, up ? a.lo : b.lo, 1 << B);
+    add(keep, other);
+    return keep;
 }
 
 // A target outside its window: validated, W taps from the row in global memory.
@@ -967,8 +984,9 @@ __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __r
         }
     };
     float* part = L.part + (size_t)g * L.M + m0;
+    float* part_lo = L.no_low ? nullptr : part + (size_t)L.S * L.M;
     fetch(warp * 32, 0);
-    float f3 = 0.0f, f4 = 0.0f, far = 0.0f;
+    Sum f3 = {0.0f, 0.0f}, f4 = f3, far = f3;
     int buf = 0;
     for (int b = warp * 32; b < ((cnt + 31) & ~31); buf ^= SUB * RS) {
         const int next = (b & 24) == 24 ? b - 24 + NW * 32 : b + SUB;
@@ -976,28 +994,29 @@ __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __r
         cp_async_wait<1>();
         __syncwarp();
         const float* r = ring + buf;
-        float f[2], all[OUT == 1 && D > 0 ? SL : 1][OUT == 1 && D > 0 ? SUB : 1];
+        Sum f[2];
+        float all[OUT == 1 && D > 0 ? SL : 1][OUT == 1 && D > 0 ? SUB : 1];
         unsigned worst = 0;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            float val[4];
+            Sum val[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int j = 4 * q + i;
                 float u[SL];
                 ring_u<D, SL>(r + j * RS, xi, lane, u);
-                val[i] = 0.0f;
 #pragma unroll
                 for (int h = 0; h < SL; ++h) {
                     unsigned rel;
                     const float t = interp_one<POLY>(u[h], first[h], nb, dump, cols + h * wstride, cf, rel);
                     worst = max(worst, rel);
-                    val[i] = h ? val[i] + t : t;
+                    if (h) add(val[i], Sum{t, 0.0f});
+                    else val[i] = {t, 0.0f};
                     if constexpr (OUT == 1 && D > 0) all[h][j] = t;
                     else if (OUT == 1) put(h, b + j, t, rel < nb);
                 }
             }
-            if (OUT == 0) f[q] = fold<1>(fold<0>(val[0], val[1], lane), fold<0>(val[2], val[3], lane), lane);
+            if (OUT == 0) f[q] = fold<1>(fold<0, SL != 1>(val[0], val[1], lane), fold<0, SL != 1>(val[2], val[3], lane), lane);
         }
         if constexpr (OUT == 1 && D > 0) {
             // eight consecutive values of the lane's slice: one 32-byte sector (U's rows are padded to 128)
@@ -1021,7 +1040,8 @@ __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __r
         }
         if (walk == 0 && __any_sync(0xffffffffu, worst >= nb)) {
             for (int i = 0; i < SUB && b + i < cnt; ++i) {
-                float u[SL], s, t = 0.0f;
+                float u[SL], s;
+                Sum t = {0.0f, 0.0f};
                 ring_u<D, SL>(r + i * RS, xi, lane, u);
 #pragma unroll
                 for (int h = 0; h < SL; ++h)
@@ -1029,18 +1049,19 @@ __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __r
                         const int ph = p + 32 * h;
                         const float q = interp_outside(L, u[h], H + (size_t)min(ph, L.P - 1) * L.G);
                         if (OUT == 1) put(h, b + i, q, true);
-                        t += q;
+                        add(t, Sum{q, 0.0f});
                     }
                 if (OUT == 0) {
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                    for (int o = 16; o > 0; o >>= 1)
+                        add(t, Sum{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
                     if (lane == ((b + i) & 31)) far = t;
                 }
             }
             __syncwarp();
         }
         if constexpr (OUT == 0) {
-            float t = fold<2>(f[0], f[1], lane);
+            Sum t = fold<2>(f[0], f[1], lane);
             if ((b & 8) == 0) {
                 f3 = t;
             } else {
@@ -1048,11 +1069,16 @@ __device__ __forceinline__ void interp_walk(const qs_launch& L, const float* __r
                 if ((b & 16) == 0) {
                     f4 = t;
                 } else {
-                    t = fold<4>(f4, t, lane) + far;
-                    far = 0.0f;
+                    t = fold<4>(f4, t, lane);
+                    add(t, far);
+                    far = {0.0f, 0.0f};
                     const int at = (b & ~31) + lane;
-                    // `more`: the group's other slices, or another walk's targets, came before
-                    if (at < cnt) part[at] = more ? part[at] + t : t;
+                    if (at < cnt) {
+                        // `more`: the group's other slices, or another walk's targets, came before
+                        if (more) add(t, Sum{part[at], part_lo ? part_lo[at] : 0.0f});
+                        part[at] = part_lo ? t.hi : t.hi + t.lo;
+                        if (part_lo) part_lo[at] = t.lo;
+                    }
                 }
             }
         }

@@ -222,7 +222,8 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     const int lane_S = qs_lane_groups(P, d, false);
     const bool ly = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, M, P, span) && (size_t)lane_S * (size_t)M * 4 <= avail;
     const bool lx = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, N, P, span);
-    const size_t need = o_part + (ly ? (size_t)lane_S : (size_t)(2 * S)) * (size_t)M * 4;
+    const bool low = (size_t)(2 * lane_S) * (size_t)M * 4 <= avail;
+    const size_t need = o_part + (ly ? (size_t)(low ? 2 * lane_S : lane_S) : (size_t)(2 * S)) * (size_t)M * 4;
     if (need > QS_NOALLOC_SCRATCH_BYTES)
         return nfail(QS_ERR_UNSUPPORTED,
                      "qs_sum_noalloc: needs %zu bytes of scratch (P=%d, G=%d, M=%lld) but the static scratch "
@@ -250,7 +251,7 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     L.S = (int)S;
     if (ly) {
         L.S = lane_S;
-        L.lane_part = true;
+        L.no_low = !low;
     }
     L.spread_variant = qs_spread_default(G, W);
 

@@ -269,7 +269,7 @@ bool grad_lane(const qs_plan p, int64_t n) { return lane_use(p, n) && (!tensor_f
 void lane_launch(const qs_plan p, qs_launch* L)
 {
     L->S = qs_lane_groups(L->P, L->d, tensor_form(p));
-    L->lane_part = true;
+    L->no_low = L->S > p->S_max;  // the partial buffer holds 2 S_max sums per target, or one per group
 }
 
 // Operand preparation of the tensor-core forms (BF16 hi/lo split or TF32
@@ -567,7 +567,7 @@ qs_status qs_plan_create(qs_plan* out, const qs_plan_desc* desc)
     QS_ALLOC(p->d_H, (size_t)P * G);
     // slice-group partials: sized for targets up to max(max_n, max_m), since the
     // gradients evaluate at x as well as at y
-    // (high and low parts of S_max groups, or sums of every 32 slices)
+    // (high and low parts of S_max groups, or more groups' sums of 32 slices without low parts)
     QS_ALLOC(p->d_part, (size_t)(2 * p->S_max > (P + 31) / 32 ? 2 * p->S_max : (P + 31) / 32) * (maxnm > 0 ? maxnm : 1));
     if (d <= QS_GRAD_MAX_D && proj == QS_PROJ_FP32_FUSED) {
         // per-component gradient partials of the fused form (the unfused forms
