@@ -172,7 +172,7 @@ qs_status qs_sum(qs_plan plan, const float* x, int64_t N, const float* w,
  * (point, slice) pair over the plan's projection buffer and back-project them
  * by a GEMM (points x P)(P x d): FP32 with compensated slice-chunk sums, or, for
  * large problems in the tensor-core forms, six products of three-way BF16
- * splits with FP32 sums over chunks of 64 slices; the fused
+ * splits with compensated sums of chunks of 64 slices; the fused
  * form, which has no projection buffer, sums the back-projection inside the
  * interpolation per component and so needs d <= 32.  x: N x d,
  * w: N (NULL = ones), y: M x d, v: M (NULL = ones), gx: N x d, gw: N,

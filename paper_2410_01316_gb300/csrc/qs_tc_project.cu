@@ -155,6 +155,21 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// The same with 16 columns.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
+{
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 template <int KIND>
 struct TcCfg;
 template <>
@@ -169,9 +184,11 @@ struct TcCfg<1> {  // TF32
 };
 
 // Back-projection, out = Q Xi: three BF16 parts of either operand, the six products down to 2^-16 of the
-// leading one.  An FP32 number has 24 bits and three parts hold them all.  114 us for 10007 targets, P =
-// 1000, d = 784 and 31 us for 30011, P = 512, d = 64, against 580 and 96 us on the FP32 pipe.  Its warps wait
-// on loads (12 of 18 warp cycles per issue); which of operands and accumulators holds them was not separated.
+// leading one.  An FP32 number has 24 bits and three parts hold them all.  111 us for 10007 targets, P =
+// 1000, d = 784 and 29 us for 30011, P = 512, d = 64, against 580 and 96 us on the FP32 pipe.  Its warps wait
+// on loads; which of operands and accumulators holds them was not separated.  Tiles of at most 128 components
+// leave room for the compensated sums and a fourth stage; 256 wide ones took 114 and 31 us there, and 10 % less of a
+// gradient at d = 200 and 256.
 template <>
 struct TcCfg<2> {
     static constexpr int ESZ = 2, BK = 32, NOPS = 3, KSTEP = 16;
@@ -180,12 +197,18 @@ struct TcCfg<2> {
 
 constexpr int ROW_BYTES = 64;               // one 64-byte swizzle row per operand row and k-slab
 constexpr int A_BYTES = TILE_M * ROW_BYTES;
-constexpr int B_BYTES = TILE_N * ROW_BYTES;
+constexpr int BACK_N = 128;                 // most components per tile of the back-projection
+
+template <int KIND>
+__host__ __device__ constexpr int b_bytes()
+{
+    return (KIND == 2 ? BACK_N : TILE_N) * ROW_BYTES;
+}
 
 template <int KIND>
 __host__ __device__ constexpr int stage_bytes()
 {
-    return TcCfg<KIND>::NOPS * (A_BYTES + B_BYTES);
+    return TcCfg<KIND>::NOPS * (A_BYTES + b_bytes<KIND>());
 }
 
 
@@ -212,8 +235,8 @@ struct PCfg<1> {  // TF32: 24 KB stages
     static constexpr int STAGES = 8;
 };
 template <>
-struct PCfg<2> {  // back-projection: 72 KB stages
-    static constexpr int STAGES = 3;
+struct PCfg<2> {  // back-projection: 48 KB stages
+    static constexpr int STAGES = 4;
 };
 
 // 32 consecutive slices (those of slice group p / 32) of point n, slice-interleaved:
@@ -240,7 +263,7 @@ constexpr int TCP_THREADS = 32 * (2 + TCP_EPI_WARPS);
 // What the back-projection (KIND 2) does besides: its inner dimension runs over the slices, 32 of a group
 // per slab (rank-3 maps of the points' parts), its columns are components in tiles of tile_n, and
 // out[n][j] = scale fac_n D[n][j] goes to row-major memory.
-constexpr int BACK_SLABS = 2;  // slabs (64 slices) per accumulator
+constexpr int BACK_SLABS = 2;  // slabs (64 slices) per accumulator (one: 5 % more of a training step at d = 784)
 struct BackArgs {
     int tile_n;
     float scale;
@@ -257,7 +280,7 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
 {
     using C = TcCfg<KIND>;
     constexpr int ST = PCfg<KIND>::STAGES;
-    constexpr int SB = stage_bytes<KIND>();
+    constexpr int SB = stage_bytes<KIND>(), B_BYTES = b_bytes<KIND>();
     extern __shared__ uint8_t smem_raw[];
     __shared__ volatile int abort_all;
     const uint32_t base = smem_u32(smem_raw);
@@ -373,15 +396,16 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
                         const uint32_t off = (uint32_t)(k * C::KSTEP * C::ESZ);
                         const uint32_t acc = (kb > k0 || k > 0) ? 1u : 0u;
                         if constexpr (KIND == 2) {
-                            // the small products first, while the sum they join is small
+                            // the leading product and the small ones, down to 2^-16 of it, in accumulators of
+                            // their own: each addition truncates its sum (see the epilogue)
                             const uint32_t id = C::IDESC + ((uint32_t)(tn / 8 - 2) << 17), a2 = a1 + A_BYTES,
-                                           b2 = b1 + B_BYTES;
-                            mma_f16(dt, sw64_desc(a2 + off), sw64_desc(b0 + off), id, acc);
-                            mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b2 + off), id, 1u);
-                            mma_f16(dt, sw64_desc(a1 + off), sw64_desc(b1 + off), id, 1u);
-                            mma_f16(dt, sw64_desc(a1 + off), sw64_desc(b0 + off), id, 1u);
-                            mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b1 + off), id, 1u);
-                            mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b0 + off), id, 1u);
+                                           b2 = b1 + B_BYTES, ds = dt + BACK_N;
+                            mma_f16(ds, sw64_desc(a2 + off), sw64_desc(b0 + off), id, acc);
+                            mma_f16(ds, sw64_desc(a0 + off), sw64_desc(b2 + off), id, 1u);
+                            mma_f16(ds, sw64_desc(a1 + off), sw64_desc(b1 + off), id, 1u);
+                            mma_f16(ds, sw64_desc(a1 + off), sw64_desc(b0 + off), id, 1u);
+                            mma_f16(ds, sw64_desc(a0 + off), sw64_desc(b1 + off), id, 1u);
+                            mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b0 + off), id, acc);
                         } else if (KIND == 0) {
                             mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b0 + off), C::IDESC, acc);
                             mma_f16(dt, sw64_desc(a0 + off), sw64_desc(b1 + off), C::IDESC, 1u);
@@ -411,16 +435,17 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
         for (int64_t t = blockIdx.x; t < T; t += gridDim.x, ++i) {
             if (abort_all) break;
             if constexpr (KIND == 2) {
-                // Each accumulator is added to FP32 sums in registers (32 of the tile's columns at a time, up
-                // to 4 times): the tensor core's own additions truncate, a bias of about 2^-25 of the running
-                // sum each, which 6 P / 16 of them in a row would make 7e-6 of the result (measured, P = 1024).
+                // Both accumulators of every 64 slices are added by TwoSum to sums in registers, 16 of the tile's
+                // columns at a time: the tensor core's own additions truncate, a bias of up to 2^-24 of the
+                // running sum each (all slices in one accumulator: 7e-6 of the result at P = 1024; the six
+                // products of 64 slices in one, and plain additions here: 1.9e-7).
                 const int half = (tn / 2 + 15) & ~15;
                 const int c0 = h * half, c1 = min(tn, c0 + half);
-                float sum[4][32];
+                float hi[4][16], lo[4][16];
 #pragma unroll
                 for (int q4 = 0; q4 < 4; ++q4)
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) sum[q4][j] = 0.0f;
+                    for (int j = 0; j < 16; ++j) hi[q4][j] = lo[q4][j] = 0.0f;
                 const int chunks = (nkb + BACK_SLABS - 1) / BACK_SLABS;
                 bool got = true;
                 for (int ch = 0; ch < chunks && got; ++ch) {
@@ -431,12 +456,16 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
                     const uint32_t trow = tmem + (uint32_t)(a * TILE_N) + ((uint32_t)(32 * q) << 16);
 #pragma unroll
                     for (int q4 = 0; q4 < 4; ++q4) {
-                        if (c0 + 32 * q4 >= c1) continue;
-                        float v[32];
+                        if (c0 + 16 * q4 >= c1) continue;
+                        float v[16];
                         __syncwarp();
-                        tmem_ld32(trow + (uint32_t)(c0 + 32 * q4), v);
+                        tmem_ld16(trow + (uint32_t)(c0 + 16 * q4), v);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) sum[q4][j] += v[j];
+                        for (int j = 0; j < 16; ++j) qs_two_sum(hi[q4][j], lo[q4][j], v[j]);
+                        __syncwarp();
+                        tmem_ld16(trow + (uint32_t)(BACK_N + c0 + 16 * q4), v);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) lo[q4][j] += v[j];
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -457,18 +486,19 @@ __global__ void __launch_bounds__(TCP_THREADS, 1)
                     const bool vec = (ldU & 3) == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
 #pragma unroll
                     for (int q4 = 0; q4 < 4; ++q4) {
-                        const int pc = p0 + c0 + 32 * q4;
-                        const int cols = min(32, min(P, p0 + c1) - pc);
+                        const int pc = p0 + c0 + 16 * q4;
+                        const int cols = min(16, min(P, p0 + c1) - pc);
                         float* o = U + (size_t)n * ldU + pc;
-                        if (cols == 32 && vec) {
+                        if (cols == 16 && vec) {
 #pragma unroll
-                            for (int j = 0; j < 32; j += 4)
-                                *reinterpret_cast<float4*>(o + j) = make_float4(sum[q4][j] * f, sum[q4][j + 1] * f,
-                                                                                sum[q4][j + 2] * f, sum[q4][j + 3] * f);
+                            for (int j = 0; j < 16; j += 4)
+                                *reinterpret_cast<float4*>(o + j) =
+                                    make_float4((hi[q4][j] + lo[q4][j]) * f, (hi[q4][j + 1] + lo[q4][j + 1]) * f,
+                                                (hi[q4][j + 2] + lo[q4][j + 2]) * f, (hi[q4][j + 3] + lo[q4][j + 3]) * f);
                         } else {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                if (j < cols) o[j] = sum[q4][j] * f;
+                            for (int j = 0; j < 16; ++j)
+                                if (j < cols) o[j] = (hi[q4][j] + lo[q4][j]) * f;
                         }
                     }
                 }
@@ -1082,10 +1112,10 @@ cudaError_t sm_count(int* out)
     return cudaSuccess;
 }
 
-// Components per tile of the back-projection: d in equal tiles of at most 256, a multiple of 16.
+// Components per tile of the back-projection: d in equal tiles of at most 128, a multiple of 16.
 int back_tile(int d)
 {
-    const int tiles = (d + TILE_N - 1) / TILE_N;
+    const int tiles = (d + BACK_N - 1) / BACK_N;
     return ((d + tiles - 1) / tiles + 15) / 16 * 16;
 }
 
