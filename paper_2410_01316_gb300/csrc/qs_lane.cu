@@ -259,7 +259,19 @@ __device__ __forceinline__ void taps_of(const Coeffs& k, float s, float (&tap)[W
 // G of them.  Windows stay inside, so that the slow way sees every other point.
 __device__ __forceinline__ int lowest_bin(int G) { return -(G >> 1) - (HW - 1); }
 
-// The bins of a sample of the points n0 .. n1 - 1, spaced evenly, into lohi:
+// A number in [0, 2^32) for sample i (the finaliser of MurmurHash3).
+__device__ __forceinline__ uint32_t sample_hash(uint32_t i)
+{
+    i = (i + 1) * 0x9E3779B9u;
+    i = (i ^ (i >> 16)) * 0x85EBCA6Bu;
+    i = (i ^ (i >> 13)) * 0xC2B2AE35u;
+    return i ^ (i >> 16);
+}
+
+// The bins of a sample of the points n0 .. n1 - 1, one at a hashed place of each
+// of NSAMPLE equal ranges (evenly spaced ones would see one cluster only of
+// points that take turns between clusters, and every other point would go the
+// slow way: 3453 against 545 us for 2 x 2e5 points, d = 16, P = 512), into lohi:
 // [h][0..31] smallest, [h][32..63] largest of each lane's slice h.  scratch:
 // NSAMPLE x D floats (the window itself, not yet in use).  All loads are issued
 // before the first is used: the sample costs one trip to memory.  Ends with a
@@ -271,8 +283,8 @@ __device__ __forceinline__ void sample_bins(const qs_launch& L, const float* __r
     constexpr int NW = NT / 32, PER = (NSAMPLE + NW - 1) / NW;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ns = (int)min(n1 - n0, (int64_t)NSAMPLE);
-    const int64_t gap = n1 - n0 > NSAMPLE ? (int64_t)((uint64_t)(n1 - n0) / NSAMPLE) : 1;  // a shift
-    auto at = [&](int i) { return n0 + i * gap; };
+    const uint32_t gap = n1 - n0 > NSAMPLE ? (uint32_t)((uint64_t)(n1 - n0) / NSAMPLE) : 1u;  // a shift; points < 2^31
+    auto at = [&](int i) { return n0 + (int64_t)i * gap + __umulhi(sample_hash((uint32_t)i), gap); };
     float us[D > 0 ? 1 : PER];
     if constexpr (D > 0) {
         for (int e = threadIdx.x; e < ns * D; e += blockDim.x) {
