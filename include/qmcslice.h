@@ -177,7 +177,13 @@ qs_status qs_sum(qs_plan plan, const float* x, int64_t N, const float* w,
  * interpolation per component and so needs d <= 32.  x: N x d,
  * w: N (NULL = ones), y: M x d, v: M (NULL = ones), gx: N x d, gw: N,
  * gy: M x d; all device memory; any output may be NULL to skip it.
- * Asynchronous on `stream`, allocates nothing.  Errors: QS_ERR_ARG,
+ * Asynchronous on `stream`.  Allocates nothing, but for the first gradient in
+ * x or y of a plan in a tensor-core form whose points on that side run with
+ * one slice per lane (qs_plan_lanes): it takes a buffer half as large as the
+ * plan's projections, under stream capture too.  If that does not fit, the
+ * plan's gradients are computed with the point-per-lane kernels and the FP32
+ * back-projection from then on: equally accurate, other last bits.
+ * Errors: QS_ERR_ARG,
  * QS_ERR_UNSUPPORTED (fused form with d > 32), QS_ERR_CUDA; data errors via
  * qs_check.
  */

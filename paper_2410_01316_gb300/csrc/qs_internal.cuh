@@ -171,9 +171,11 @@ struct qs_plan_s {
     // directions hi/lo (128-row boxes, the SM-pair kernel)
     alignas(64) unsigned char tmaps[6][128];
     alignas(64) unsigned char tmaps_y[6][128];  // the same with the targets' staging as A
-    // back-projection GEMM of the tensor-core forms: low parts of the derivative values, directions
-    // transposed and split (NULL: not available, the SIMT back-projection is used)
+    // back-projection GEMM of the tensor-core forms: low parts of the derivative values (taken by the first
+    // gradient; NULL afterwards: did not fit, the SIMT back-projection is used), directions transposed and
+    // split (NULL: no number of points of this plan takes the GEMM)
     void* d_qlo;
+    bool qlo_tried;
     void* d_xit;
     alignas(64) unsigned char tmaps_q[6][128];
     bool gemm_pair;       // projection GEMM on SM pairs (cta_group::2)

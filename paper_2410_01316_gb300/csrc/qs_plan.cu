@@ -262,8 +262,32 @@ bool lane_use(const qs_plan p, int64_t n)
 
 bool tensor_form(const qs_plan p) { return p->proj == QS_PROJ_BF16X3 || p->proj == QS_PROJ_TF32; }
 
-// The same for the targets of a gradient, which the tensor-core forms back-project from BF16 parts.
-bool grad_lane(const qs_plan p, int64_t n) { return lane_use(p, n) && (!tensor_form(p) || p->d_qlo); }
+// The same for the targets of a gradient, deriv: of derivative values, which the tensor-core forms back-project
+// from BF16 parts.
+bool grad_lane(const qs_plan p, int64_t n, bool deriv) { return lane_use(p, n) && (!(tensor_form(p) && deriv) || p->d_qlo); }
+
+int ldq_of(int P) { return (P + 7) / 8 * 8; }
+
+// The buffer of the derivative values' low parts, half as large as U: taken by the first gradient whose
+// targets run slice-per-lane, so that plans which only sum do without it.  Where it does not fit (tried once)
+// the plan's gradients keep the point-per-lane kernels and the FP32 back-projection.  The allocation is in order
+// under stream capture too, this thread's or another's: in the relaxed mode it does not disturb either.
+void grad_buffers(const qs_plan p)
+{
+    if (p->d_qlo || p->qlo_tried || !p->d_xit) return;
+    p->qlo_tried = true;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return;
+    uint16_t* ql = nullptr;
+    if (dalloc(&ql, (size_t)((p->desc.P + 31) / 32) * (size_t)p->ldU * 32) != cudaSuccess) {
+        cudaGetLastError();
+    } else if (qs_make_backproj_maps(p->tmaps_q, p->d_U, ql, p->d_xit, p->ldU, p->desc.P, p->desc.d, ldq_of(p->desc.P))) {
+        p->d_qlo = ql;
+    } else {
+        cudaFree(ql);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+}
 
 // The launch of the slice-per-lane interpolation and of the reduction after it.
 void lane_launch(const qs_plan p, qs_launch* L)
@@ -623,6 +647,11 @@ qs_status qs_plan_create(qs_plan* out, const qs_plan_desc* desc)
         QS_ALLOC(yh, (size_t)ystage_rows * p->ldk);
         p->d_ys_hi = yh;
     }
+    if (tc && lane_use(p, maxnm)) {
+        uint16_t* xt = nullptr;
+        QS_ALLOC(xt, (size_t)3 * d * ldq_of(P));
+        p->d_xit = xt;
+    }
     QS_ALLOC(p->d_x, (size_t)(D.max_n > 0 ? D.max_n : 1) * d);
     QS_ALLOC(p->d_w, (size_t)(D.max_n > 0 ? D.max_n : 1));
     QS_ALLOC(p->d_y, (size_t)(D.max_m > 0 ? D.max_m : 1) * d);
@@ -688,25 +717,9 @@ qs_status qs_plan_create(qs_plan* out, const qs_plan_desc* desc)
         for (int i = 0; i < 4; ++i)
             QS_CHECK(cudaEventCreateWithFlags(&p->sev[i], i < 2 ? cudaEventDisableTiming : cudaEventDefault),
                      "fork / join events");
-        // back-projection GEMM: its buffers only make gradients faster, so a plan does without where they
-        // do not fit
-        if (W == QS_LANE_W) {
-            const size_t groups = (P + 31) / 32;
-            const int ldq = (P + 7) / 8 * 8;
-            uint16_t *ql = nullptr, *xt = nullptr;
-            bool okq = dalloc(&ql, groups * (size_t)p->ldU * 32) == cudaSuccess;
-            p->d_qlo = ql;
-            okq = okq && dalloc(&xt, (size_t)3 * d * ldq) == cudaSuccess;
-            p->d_xit = xt;
-            okq = okq && qs_make_backproj_maps(p->tmaps_q, p->d_U, ql, xt, p->ldU, P, d, ldq) &&
-                  qs_launch_split_xit(p->d_dirs, P, d, ldq, xt, 0) == cudaSuccess;
-            if (!okq) {
-                cudaGetLastError();
-                cudaFree(p->d_qlo);
-                cudaFree(p->d_xit);
-                p->d_qlo = p->d_xit = nullptr;
-            }
-        }
+        // directions of the back-projection GEMM (its other buffer waits for the first gradient)
+        if (p->d_xit)
+            QS_CHECK(qs_launch_split_xit(p->d_dirs, P, d, ldq_of(P), p->d_xit, 0), "split of the transposed directions");
         // the SM-pair GEMM where the GEMM is tensor-bound (d >= 256: 6 d flop
         // per 4 B of U written) and two-CTA clusters of it can be resident;
         // below, the U stores bound both forms and the single-SM one is faster
@@ -968,6 +981,7 @@ qs_status qs_grad(qs_plan p, const float* x, int64_t N, const float* w, const fl
     const int d = p->desc.d;
     const float scale = (float)(p->tau / (double)p->desc.P);
     const bool fused = p->proj == QS_PROJ_FP32_FUSED, from_u = tensor_form(p);
+    if (from_u && ((gy && lane_use(p, M)) || (gx && lane_use(p, N)))) grad_buffers(p);
     // Sources -> grids: plain (into d_H) and / or derivative (into d_H2).
     auto grids = [&](const qs_launch& L, const float* pts, const float* wt, bool plain, bool deriv) {
         const bool lane = lane_use(p, L.N);
@@ -985,7 +999,7 @@ qs_status qs_grad(qs_plan p, const float* x, int64_t N, const float* w, const fl
     };
     // Plain values of the grids at the targets (projected already where the form is unfused), summed over slices.
     auto values = [&](qs_launch L, const float* pts, float* out) {
-        const bool lane = fused ? lane_use(p, L.M) : grad_lane(p, L.M);
+        const bool lane = grad_lane(p, L.M, gx != nullptr);  // one projection for both
         if (lane) lane_launch(p, &L);
         cudaError_t e = lane ? qs_launch_lane_interp(L, pts, from_u, p->d_H, false, st)
                              : qs_launch_interp(L, p->W, pts, fused, st);
@@ -1001,7 +1015,7 @@ qs_status qs_grad(qs_plan p, const float* x, int64_t N, const float* w, const fl
             e = qs_launch_interp_grad(L, p->W, pts, p->d_H2, p->d_dirs, p->d_gpart, fused, st);
             return e == cudaSuccess ? qs_launch_reduce_grad(p->d_gpart, L.S, L.M, d, scale, fac, out, st) : e;
         }
-        if (!grad_lane(p, L.M)) {
+        if (!grad_lane(p, L.M, true)) {
             cudaError_t e1 = qs_launch_interp_deriv(L, p->W, p->d_H2, st);
             return e1 == cudaSuccess ? qs_launch_backproj(p->d_U, p->ldU, L.M, L.P, p->d_dirs, d, scale, fac, out, st) : e1;
         }
@@ -1019,7 +1033,7 @@ qs_status qs_grad(qs_plan p, const float* x, int64_t N, const float* w, const fl
         } else {
             const qs_launch L = make_launch(p, N, M, 256);
             e = grids(L, x, w, false, true);
-            if (e == cudaSuccess && !fused) e = project(p, y, M, st, grad_lane(p, M));
+            if (e == cudaSuccess && !fused) e = project(p, y, M, st, grad_lane(p, M, true));
             if (e == cudaSuccess) e = gradient(L, y, v, gy);
         }
         if (e != cudaSuccess) return cuda_fail(e, "qs_grad: gradient in y");
@@ -1035,7 +1049,7 @@ qs_status qs_grad(qs_plan p, const float* x, int64_t N, const float* w, const fl
             // gets the slice-group count matching its CTA shape
             const qs_launch L = make_launch(p, M, N, 256);
             e = grids(L, y, v, gw != nullptr, gx != nullptr);
-            if (e == cudaSuccess && !fused) e = project(p, x, N, st, grad_lane(p, N));
+            if (e == cudaSuccess && !fused) e = project(p, x, N, st, grad_lane(p, N, gx != nullptr));
             // the plain interpolation reads the projections before the
             // derivative values overwrite them
             if (e == cudaSuccess && gw) e = values(make_launch(p, M, N, 256 * qs_interp_tpt(fused, d, p->G)), x, gw);
