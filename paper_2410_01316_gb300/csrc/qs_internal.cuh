@@ -375,9 +375,19 @@ inline bool qs_lane_use(qs_proj proj, int W, int d, int64_t n, int P, double spa
     // them their results: with few slices to average over, the two kinds differ by the rounding of the
     // point-per-lane spread to sum |w| 2^-30, up to 3e-5 of a result whose weights cancel.
     if (P <= QS_LANE_FEW && n < QS_LANE_FEW_POINTS) return false;
-    // placing, clearing and adding up the windows takes 10 to 30 us, the more the more coordinates a lane
-    // holds: even with the point-per-lane kernels at 1e6 pairs with projections from U or d <= 4 (d = 64:
-    // 78 us either way; at 2e6 84 against 88), 4e6 at d = 16, 6e6 at d = 30
-    const int64_t least = proj == QS_PROJ_BF16X3 || proj == QS_PROJ_TF32 || d <= 4 ? 2 << 20 : (d <= 16 ? 3 << 20 : 6 << 20);
+    // Placing, clearing and adding up the windows takes 10 to 30 us, the more the more coordinates a lane holds.
+    // Speed of a sum of n sources and n targets against the point-per-lane kernels, at n P =
+    //                       2.05        3.1            4.0            5.0            6.5 (x 2^20)
+    //   d = 3  P = 320      0.96        1.07           1.20           1.33           1.52
+    //          P = 640      1.00        1.10           1.17           1.23           1.42
+    //   d = 5, 8, 16  320    -          1.01 to 1.12   1.12 to 1.16   1.20 to 1.23   1.27 to 1.30
+    //                 640    -          1.20 to 1.28   1.14 to 1.20   1.13 to 1.17   1.30 to 1.32
+    //   d = 30 P = 320       -            -              -              -            1.07
+    //   d = 64 P = 320      0.92        1.03           1.05           1.12           1.17
+    //   (BF16x3)    640     1.01        1.14           1.11           1.10           1.23
+    // From P = 1280 on it is 1.17 to 1.4 wherever a value stands, at P = 4096 (n from 512) 1.7 to 2.5.  At the lower line of
+    // a row the targets gain more (1.03 to 1.35) than the sources (0.93 to 1.03).
+    int64_t least = proj == QS_PROJ_BF16X3 || proj == QS_PROJ_TF32 || d <= 4 ? 2 << 20 : (d <= 16 ? 3 << 20 : 6 << 20);
+    if (P < 512 && least < 3 << 20) least = 3 << 20;
     return n >= 512 && n < ((int64_t)1 << 31) && n * (int64_t)P >= least;
 }
