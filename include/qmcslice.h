@@ -280,7 +280,7 @@ qs_status qs_stage_times(qs_plan plan, float* ms, int n);
  * allocation, or plugins that are handed their buffers and nothing else.
  * Plan creation allocates, so they cannot hold a plan.  qs_sum_noalloc takes
  * the plan description directly and keeps every intermediate in one static
- * device array of 16 MiB that the library reserves on each GPU it is loaded
+ * device array of 16 MiB (and 1 KB) that the library reserves on each GPU it is loaded
  * on, until the process exits.  It allocates nothing.
  *
  * desc: as for qs_plan_create; dirs, seed, dirs_host, max_n and max_m are

@@ -12,8 +12,9 @@
 // (d <= 64), but every intermediate -- the filter table, the twiddles, the
 // scaled directions, the per-slice filtered grids, the slice partial sums,
 // the weight scale and the error flag -- lives in one file-scope device
-// array of QS_NOALLOC_SCRATCH_BYTES (16 MiB).  Every GPU that loads the
-// library holds that array until the process exits.  No call allocates.
+// array of QS_NOALLOC_SCRATCH_BYTES (16 MiB and the partials of the weight
+// bound).  Every GPU that loads the library holds that array until the process
+// exits.  No call allocates.
 //
 // Sharing: all calls on a device use the same array and it keeps the last
 // call's contents; each call rewrites everything it reads (the error flag is
@@ -33,7 +34,9 @@
 
 #include "qs_internal.cuh"
 
-#define QS_NOALLOC_SCRATCH_BYTES (16u << 20)
+// the partials of the weight bound (1024 B beyond the two values of the smaller kernels) come on top of the
+// 16 MiB, so that every problem that fits those without them still runs
+#define QS_NOALLOC_SCRATCH_BYTES ((16u << 20) + 1024u)
 #define QS_NOALLOC_MAX_DEVICES 64
 #define QS_NOALLOC_TABLE_CACHE 4
 
@@ -209,6 +212,8 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     if (S > S_max) S = S_max;
     if (S < 1) S = 1;
     const size_t o_flag = 0, o_wscale = 256, o_psihat = o_wscale + align256(QS_WSCALE_FLOATS * 4);
+    static_assert(256 + (QS_WSCALE_FLOATS * 4 + 255) / 256 * 256 == 512 + (QS_NOALLOC_SCRATCH_BYTES - (16u << 20)),
+                  "the array grows by what the partials take");
     const size_t o_c = o_psihat + align256((size_t)(K + 1) * 8);
     const size_t o_D = o_c + align256((size_t)D.n_ft * 8);
     const size_t o_tw = o_D + align256((size_t)(G / 2 + 1) * 4);
@@ -222,7 +227,7 @@ extern "C" qs_status qs_sum_noalloc(const qs_plan_desc* desc, const float* dirs_
     const int lane_S = qs_lane_groups(P, d, false);
     const bool ly = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, M, P, span) && (size_t)lane_S * (size_t)M * 4 <= avail;
     const bool lx = qs_lane_use(QS_PROJ_FP32_FUSED, W, d, N, P, span);
-    const bool low = (size_t)(2 * lane_S) * (size_t)M * 4 <= avail;
+    const bool low = lane_S <= S_max && (size_t)(2 * lane_S) * (size_t)M * 4 <= avail;  // as a plan has them
     const size_t need = o_part + (ly ? (size_t)(low ? 2 * lane_S : lane_S) : (size_t)(2 * S)) * (size_t)M * 4;
     if (need > QS_NOALLOC_SCRATCH_BYTES)
         return nfail(QS_ERR_UNSUPPORTED,
