@@ -232,11 +232,7 @@ def run_ours(args, rank, world, local_rank):
     stream = torch.cuda.current_stream()
     flush = torch.empty(64 * 1024 * 1024, dtype=torch.float32, device=dev)  # 256 MB > 129 MB L2
 
-    if args.spread_variant:
-        plan.set_variant(args.spread_variant)
-        spread_variant = args.spread_variant
-    else:
-        spread_variant = plan.autotune(x, w)
+    spread_variant = tuned_variant(plan, x, w, args.spread_variant)
     if args.gemm != "auto" and plan.proj in ("bf16x3", "tf32"):
         plan.set_gemm(args.gemm == "pair")
     gemm = ("pair" if plan.gemm_pair() else "single") if plan.proj in ("bf16x3", "tf32") else None
@@ -325,7 +321,7 @@ def run_ours(args, rank, world, local_rank):
             "e2e": {"value": ps_step * args.steps * world / e2e_t / 1e9, "unit": UNIT,
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "ms_per_step": 1e3 * e2e_t / args.steps},
-            "gpu_launches": args.steps * launches_per_step(plan),
+            "gpu_launches": args.steps * launches_per_step(plan, prob.N, prob.M),
         }
         if proj != "fp32" and not args.no_fp32_compare:
             line["config"]["plain_fp32"] = plain_fp32_compare(prob, x, w, y, flush, args, err_idx_err=not args.no_error_check)
@@ -539,7 +535,7 @@ def precision_forms(args, flush, clocks, peaks, peak_src, sm_count):
     for form in ("fp32", "tf32", "bf16x3", "fp32_fused"):
         with QSPlan(prob.d, prob.kernel, prob.P, prob.n_ft, prob.R, prob.kparam, dirs=prob.xi, window=prob.window,
                     proj=form, max_n=prob.N, max_m=prob.M) as plan:
-            variant = plan.autotune(x, w)
+            variant = tuned_variant(plan, x, w)
             gemm = ("pair" if plan.gemm_pair() else "single") if form in ("bf16x3", "tf32") else None
             for _ in range(max(3, args.warmup)):
                 plan.sum(x, w, y, out=s)
@@ -561,16 +557,16 @@ def precision_forms(args, flush, clocks, peaks, peak_src, sm_count):
             status = plan.status()
             stages = {k: v / steps for k, v in stage_acc.items()}
             _, rl = roofline(prob, plan, stages, clocks, peaks, peak_src, sm_count)
+            u_rt = sum(8.0 * n * prob.P for n in (prob.N, prob.M) if projects(plan, n))
         with QSPlan(prob.d, prob.kernel, n_sub, prob.n_ft, prob.R, prob.kparam, dirs=prob.xi[:n_sub],
                     window=prob.window, proj=form, max_n=prob.N, max_m=prob.M) as sp:
             sp.sum(x, w, y, out=s)
             sp.check()
             err = float(np.max(np.abs(s.cpu().numpy().astype(np.float64)[idx] - ref))) / norm
         t = sum(ms) / len(ms)
-        # HBM bytes the form must move: inputs and output, plus, unfused, the projection buffer
-        # written by the GEMM and read by the spread and interpolation (4 B per point-slice each way)
+        # HBM bytes the form must move: inputs and output, plus, where the points are projected ahead, the projection
+        # buffer written by the GEMM and read by the spread and interpolation (4 B per point-slice each way)
         io = 4.0 * ((prob.N + prob.M) * prob.d + prob.N + prob.M)
-        u_rt = 0.0 if form == "fp32_fused" else 8.0 * (prob.N + prob.M) * prob.P
         out["forms"][form] = {
             "ms_per_step": t, "value": prob.point_slices / (t / 1e3) / 1e9, "unit": UNIT,
             "hbm_bytes_inputs_outputs": io, "hbm_bytes_projection_round_trip": u_rt,
@@ -668,7 +664,7 @@ def run_gpu_compare(args, rank, world, local_rank):
         s = torch.empty(prob.M, dtype=torch.float32, device=dev)
         with QSPlan(prob.d, prob.kernel, prob.P, prob.n_ft, prob.R, prob.kparam, dirs="distance", seed=7,
                     window=prob.window, proj="auto", max_n=prob.N, max_m=prob.M, kparam2=prob.kparam2) as plan:
-            variant = plan.autotune(x, w)
+            variant = tuned_variant(plan, x, w)
             for _ in range(max(3, args.warmup)):
                 plan.sum(x, w, x, out=s)
             plan.check()
@@ -1043,7 +1039,7 @@ def run_batch(args, rank, world, local_rank, emit=True):
         sb = torch.empty(big.M, device=dev)
         with QSPlan(big.d, big.kernel, big.P, big.n_ft, big.R, big.kparam, dirs=big.xi, proj="auto", max_n=big.N,
                     max_m=big.M) as bp:
-            bp.autotune(xb, wb)
+            tuned_variant(bp, xb, wb)
             for _ in range(3):
                 bp.sum(xb, wb, yb, out=sb)
             tb = []
@@ -1084,12 +1080,27 @@ def run_batch(args, rank, world, local_rank, emit=True):
     return line
 
 
-def launches_per_step(plan) -> int:
-    # [split x,] projection x, weight bound and cleared grids, spread, filter, [split y,] projection y,
-    # interpolation, reduction (the benchmark's sizes run slice-per-lane)
-    if plan.proj in ("bf16x3", "tf32"):
-        return 9
-    return 7 if plan.proj == "fp32" and plan.d > 64 else 5
+def projects(plan, n) -> bool:
+    """Whether n points are projected by kernels of their own: not in the fused form, nor in the FP32 form where the
+    grid kernels with one slice per lane do it."""
+    return plan.proj in ("bf16x3", "tf32") or (plan.proj == "fp32" and not plan.lanes(n))
+
+
+def tuned_variant(plan, x, w, fixed=""):
+    """Spread variant in use: the one asked for, else the fastest; none where the spread has no variants."""
+    if fixed:
+        plan.set_variant(fixed)
+    elif not plan.lanes(x.shape[0]):
+        return plan.autotune(x, w)
+    return "slice per lane" if plan.lanes(x.shape[0]) else fixed
+
+
+def launches_per_step(plan, N, M) -> int:
+    """Kernel launches of one sum: [split and] projection of either side, [weight bound,] spread and filter, or
+    weight bound with cleared grids, spread, filter; interpolation, reduction."""
+    per_side = 2 if plan.proj in ("bf16x3", "tf32") else 1
+    spread = 3 if plan.lanes(N) else (1 if N <= 4096 else 2)
+    return per_side * (projects(plan, N) + projects(plan, M)) + spread + 2
 
 
 # DRAM bytes (read + write) per launch from one ncu capture of the default workload itself
@@ -1122,9 +1133,7 @@ def stage_rooflines(prob, plan, stages, clocks, peaks, peak_src, sm_count):
 
     for name, rows in (("project_x", N), ("project_y", M)):
         t = stages.get(name, 0.0) / 1e3
-        # the fused form, and the FP32 form of large problems, project inside the spread and interpolation:
-        # no kernel runs in this stage (an empty stage is a few microseconds)
-        if t <= 0 or plan.proj == "fp32_fused" or (plan.proj == "fp32" and 2.0 * rows * P * d / t / 1e12 > 1.5 * fp32_peak):
+        if t <= 0 or not projects(plan, rows):  # no kernel runs in this stage
             continue
         if plan.proj == "bf16x3":
             fl = 6.0 * rows * P * d
@@ -1147,7 +1156,6 @@ def stage_rooflines(prob, plan, stages, clocks, peaks, peak_src, sm_count):
         by = rows * d * 8.0  # read FP32, write BF16 hi + lo (or TF32)
         add(name, "hbm", by / t / 1e9, peaks["hbm_gbs"], "GB/s", f"8 B per coordinate = {by:.3e} B",
             f"hbm_gbs ({peak_src})")
-    unfused = plan.proj in ("bf16x3", "tf32") or "project_x" in out
 
     def hbm(name, by, what):
         # the same stage against HBM: its algorithmic byte stream
@@ -1164,7 +1172,7 @@ def stage_rooflines(prob, plan, stages, clocks, peaks, peak_src, sm_count):
         t = stages.get(name, 0.0) / 1e3
         if t <= 0:
             continue
-        if unfused:
+        if projects(plan, rows):
             add(name, "hbm", by / t / 1e9, peaks["hbm_gbs"], "GB/s", f"{what} = {by:.3e} B", f"hbm_gbs ({peak_src})")
             hbm(name, by, what)
         else:
