@@ -1244,8 +1244,10 @@ __global__ void __launch_bounds__(interp_threads(D), 1)
     }
 }
 
-// Dynamic shared memory of a CTA: all that the static 256 bytes leave.
+// Dynamic shared memory of a CTA: whole KB of the 227 that the kernels' static arrays leave (sampled bins of
+// two slices per lane, coefficients, a float per warp).
 constexpr int LANE_SMEM = 226 * 1024;
+static_assert(LANE_SMEM + 64 * 2 * 4 + HW * T4 * 8 + 32 * 4 <= 227 * 1024, "static and dynamic shared memory of a CTA");
 
 // How the work is cut: `group` units in each of `groups` slice groups, at least `least` per CTA; `visit` units
 // cost as much as placing, clearing and adding up a window.  A range of equal shares crosses into a second

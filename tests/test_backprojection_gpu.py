@@ -72,3 +72,10 @@ def test_every_tile_against_64_bits(d, P, M):
     x, w, y, xi = _inputs(d, P, M, 1)
     ref = _grad64(x, w, y, xi, 16.0, 512)
     assert float((_grad(x, w, y, xi, "bf16x3") - ref).abs().max()) < 2e-6 * float(ref.abs().max())
+
+
+def test_tf32_and_bf16x3_give_the_same_bits_from_the_same_projections():
+    import torch
+
+    x, w, y, xi = _inputs(64, 1000, 7003, 2)  # 11 bits hold every coordinate
+    assert torch.equal(_grad(x, w, y, xi, "tf32"), _grad(x, w, y, xi, "bf16x3"))
