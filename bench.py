@@ -654,7 +654,7 @@ def run_gpu_compare(args, rank, world, local_rank):
     flush = torch.empty(64 * 1024 * 1024, dtype=torch.float32, device=dev)
     stream = torch.cuda.current_stream()
     kernels = ("gauss", "laplace", "matern", "negdist")
-    per, tot_ps, tot_ms = {}, 0, 0.0
+    per, tot_ps, tot_ms, launches = {}, 0, 0.0, 0
     sampler = ClockSampler(smi_gpu_id(dev))
     sampler.start()
     for kern in kernels:
@@ -681,6 +681,7 @@ def run_gpu_compare(args, rank, world, local_rank):
             status = plan.status()
             xi = plan.directions()
             proj = plan.proj
+            launches += args.steps * launches_per_step(plan, prob.N, prob.N)
         t = sum(ms) / len(ms)
         tot_ps += prob.point_slices
         tot_ms += t
@@ -714,7 +715,7 @@ def run_gpu_compare(args, rank, world, local_rank):
                                    "coordinates) summed against themselves, w = 1, P=5120 distance QMC directions, "
                                    "median rule; one step = the Gauss, Laplace, Matern and negative distance sums",
                        "kernels": per, "l2": "flushed between steps (256 MB write); inputs also exceed L2"},
-            "clocks": clocks, "gpu_launches": args.steps * 4 * 6}
+            "clocks": clocks, "gpu_launches": launches}
     if rank == 0:
         print(json.dumps(line), flush=True)
 
@@ -875,7 +876,8 @@ def run_mmd_flow(args, rank, world, local_rank, emit=True):
                                    f"negdist, N_ft={n_ft}, Euler h={h} on M grad (gradient over {N + M} sources)",
                        "mmd2_curve": curve, "device_status": int(status),
                        "point_slices_per_step": f"(N + M sources + M targets) P = {ps}"},
-            "clocks": clocks, "gpu_launches": args.steps * 4}
+            # projections, weight bound, derivative grids (spread and filter), values, back-projection
+            "clocks": clocks, "gpu_launches": args.steps * (projects(plan, N + M) + projects(plan, M) + (3 if plan.lanes(N + M) else 2) + 2)}
     if rank == 0 and emit:
         print(json.dumps(line), flush=True)
     plan.close()
@@ -1107,7 +1109,7 @@ def launches_per_step(plan, N, M) -> int:
 # (d = 784, N = M = 60000, P = 2048, N_ft = 1024, BF16x3 on the SM-pair GEMM, slice-per-lane
 # spread and interpolation; profiles/traffic_mnist_laplace.md).  Only for that configuration and
 # the kernels as captured.
-TRAFFIC_MNIST = {"project_x": 639.6e6, "project_y": 637.1e6, "spread_filter": 512.7e6, "interp": 509.4e6}
+TRAFFIC_MNIST = {"project_x": 640.6e6, "project_y": 637.0e6, "spread_filter": 512.7e6, "interp": 522.1e6}
 
 
 def _traffic(prob, plan, name):

@@ -20,15 +20,16 @@
 // more than the shared memory holds, the points are walked once per window.
 //
 // No unit is full: 2.0 to 3.0 of 4 warp instructions a clock, the load / store
-// pipe at 36 to 79 %, FP32 at 26 to 40 %.  Warp instructions per 32 point-slices,
-// projection included where it is done here: spread 52 (moments, U read) to 87
-// (cells, d = 16), interpolation 37 (polynomials, U read) to 73 (derivative, d = 16).
+// pipe at 36 to 71 %, FP32 at 28 to 40 %.  Warp instructions per 32 point-slices,
+// projection included where it is done here: spread 53 (moments, U read) to 92
+// (cells, d = 16), interpolation 47 (polynomials, U read; 10 of them the compensated
+// sums) to 74 (derivative, d = 16).
 // Kernel times against the kernels with one point per lane (us):
-//   spread         d = 784, 6e4 points, P = 2048, G = 2048    822 (one kernel with the filter) -> 216 + 29
-//                  d = 64, 2e5, P = 1024, G = 4096            814 -> 509 + 31
-//                  d = 30, 9.6e5, P = 1280, G = 256           7590 + 2123 (projection) -> 3520 + 8
-//                  d = 16, 2e5, P = 1024, G = 2048            740 and a projection (316 with that of y) -> 696 + 17
-//   interpolation  d = 784  344 -> 171   d = 64  867 -> 462   d = 30  3180 + 2129 -> 2970
+//   spread         d = 784, 6e4 points, P = 2048, G = 2048    822 (one kernel with the filter) -> 215 + 34
+//                  d = 64, 2e5, P = 1024, G = 4096            814 -> 537 + 39
+//                  d = 30, 9.6e5, P = 1280, G = 256           7590 + 2123 (projection) -> 3608 + 8
+//                  d = 16, 2e5, P = 1024, G = 2048            740 and a projection (316 with that of y) -> 712 + 20
+//   interpolation  d = 784  344 -> 203   d = 64  867 -> 525   d = 30  3180 + 2129 -> 3143
 #include <cuda_bf16.h>
 #include <float.h>
 #include <limits.h>

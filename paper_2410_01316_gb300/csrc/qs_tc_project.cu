@@ -185,8 +185,8 @@ struct TcCfg<1> {  // TF32
 
 // Back-projection, out = Q Xi: three BF16 parts of either operand, the six products down to 2^-16 of the
 // leading one.  An FP32 number has 24 bits and three parts hold them all.  111 us for 10007 targets, P =
-// 1000, d = 784 and 29 us for 30011, P = 512, d = 64, against 580 and 96 us on the FP32 pipe.  Its warps wait
-// on loads; which of operands and accumulators holds them was not separated.  Tiles of at most 128 components
+// 1000, d = 784 and 29 us for 30011, P = 512, d = 64, against 580 and 96 us on the FP32 pipe.  1.7 of 4
+// warp instructions a clock; the epilogue's warps wait on loads of the accumulators (2.3 of 5.7 cycles per issue).  Tiles of at most 128 components
 // leave room for the compensated sums and a fourth stage; 256 wide ones took 114 and 31 us there, and 10 % less of a
 // gradient at d = 200 and 256.
 template <>
